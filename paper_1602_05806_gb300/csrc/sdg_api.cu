@@ -218,6 +218,43 @@ int cg_loop(sdg_handle* h, const Op& op, T* x, T* const* r, T* const* p, T* cons
   return SDG_OK;
 }
 
+// Iterations of one segment in the resident kernel: until the device pauses or
+// stops the solve, or segment_cap iterations.  Buffers and x as in the
+// one-launch form of cg_loop.  The caller reads the state back and advances
+// the tag by the iterations done plus one (resident_sync).
+template <typename T>
+int cg_resident(sdg_handle* h, const Op& op, const ResPlan& pl, T* x, T* const* r, T* const* p, T* const* Ap, int sid,
+                cudaStream_t s, long long segment_cap, double delta2) {
+  ResArgs<T> a{};
+  for (int k = 0; k < 2; ++k) {
+    a.r[k] = r[k];
+    a.p[k] = p[k];
+    a.ap[k] = Ap[k];
+  }
+  a.x = x;
+  for (int d = 0; d < 3; ++d) a.s[d] = op.s[d];
+  a.cmass = op.cmass;
+  a.st = st_dev(h, sid);
+  a.tag = h->res_tag;
+  a.cap = (int)std::min<long long>(segment_cap, h->maxit);
+  a.delta2 = delta2;
+  SDG_K(h->dim == 2 ? res_dispatch_2d(h, pl, a, s) : res_dispatch_3d(h, pl, a, s));
+  return SDG_OK;
+}
+
+// The state after a resident segment (and what was launched behind it).
+int resident_sync(sdg_handle* h, int sid, cudaStream_t s) {
+  const int it0 = h->st_host[sid].iter;
+  SDG_CK(cudaMemcpyAsync(h->st_host + sid, st_dev(h, sid), sizeof(SolverState), cudaMemcpyDeviceToHost, s));
+  SDG_CK(cudaStreamSynchronize(s));
+  h->res_tag += (unsigned)(h->st_host[sid].iter - it0) + 1u;
+  if (h->st_host[sid].status == SDG_ERR_CUDA) {
+    set_err("a wait of the resident CG kernel ran out%s", "");
+    return SDG_ERR_CUDA;
+  }
+  return SDG_OK;
+}
+
 void fill_info(sdg_cg_info* info, const SolverState& hs, int outer, int a64, int a32, int status,
                double true_res, double floor_res, double eval_res) {
   if (status != SDG_OK) {
@@ -309,44 +346,85 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   double* pa = parts(h, sid);
   const double delta = h->delta;
   const int unscaled = fp32 ? 0 : 1;
-  // one launch per iteration unless asked otherwise or the FP32 iteration
-  // deflates the kernel
-  const bool fused = !deflate && h->form == 0;
+  // the default form on grids whose tiles fit the GPU at once: the resident
+  // kernel, which runs the one-launch form's iteration (with every launch to
+  // be timed, or a tile shape asked for, the iterations stay single launches);
+  // its replacements are one launch too where the FP64 tiles fit (whole)
+  const ResPlan& plan = h->res[fp32 ? 1 : 0];
+  const bool resident = !deflate && h->form == 2 && h->tile32 == 0 && !h->profile && plan.state == 1;
+  const bool whole = resident && h->res[0].state == 1;
+  // one launch per iteration or less unless asked otherwise or the FP32
+  // iteration deflates the kernel
+  const bool fused = resident || (!deflate && h->form == 0);
   double* r64v[2] = {h->r64, fused ? h->r64b : h->r64};
   double* Ap64v[2] = {h->Ap64, fused ? h->Ap64b : h->Ap64};
   float* r32v[2] = {h->r32, fused ? h->r32b : h->r32};
   float* Ap32v[2] = {h->Ap32, fused ? h->Ap32b : h->Ap32};
   int a64 = 0, updates = 0;
-  if (singular) SDG_CK(cudaMemcpyAsync(h->x0buf, x, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  // start: r = b - A x0 (x32 = 0)
-  if (fp32) SDG_CK(cudaMemsetAsync(h->x32, 0, n * sizeof(float), s));
-  SDG_K(apply_plain<double>(h, op, x, h->Ap64, s, 1));
-  ++a64;
-  SDG_K(rel_residual(b, h->Ap64, h->r64, n, st, pa, rtol, h->maxit, fp32 ? delta : 0.0, 1, singular, unscaled, s));
-  if (singular) {
-    int nl = 0;
-    SDG_CK(kernel_restore(h, h->r64, nullptr, s, &nl));
-    h->launches += nl;
-    SDG_K(rel_renorm(h->r64, n, st, pa, 1, s));
-  }
-  SDG_CK(cudaMemcpyAsync(h->st_host + sid, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
-  SDG_CK(cudaStreamSynchronize(s));
-  // the reachable tolerance: three times the FP64 residual floor near x0
   double floor_res = 0.0;
-  if (!h->st_host[sid].done) {
-    const int rc = floor_residual(h, op, x, h->st_host[sid].bnorm2, singular, s, &floor_res);
-    if (rc != SDG_OK) return rc;
-    ++a64;
-    if (3.0 * floor_res > rtol) {
-      SolverState& hs = h->st_host[sid];
-      const double tol = 3.0 * floor_res;
-      hs.tol2 = tol * tol * hs.bnorm2 * hs.sigma * hs.sigma;
-      if (hs.rr <= hs.tol2) hs.done = 1;
-      SDG_CK(cudaMemcpyAsync(st, h->st_host + sid, sizeof(SolverState), cudaMemcpyHostToDevice, s));
+  ResidArgs rsd{};  // start and replacements of a whole resident solve
+  auto resid = [&](int start) -> int {
+    rsd.start = start;
+    rsd.tag = h->resid_tag;
+    h->resid_tag += 3u;
+    SDG_K(h->dim == 2 ? resid_dispatch_2d(h, h->res[0], rsd, s) : resid_dispatch_3d(h, h->res[0], rsd, s));
+    return SDG_OK;
+  };
+  if (whole) {
+    rsd.b = b;
+    rsd.x = x;
+    rsd.x0 = h->x0buf;
+    rsd.x32 = fp32 ? h->x32 : nullptr;
+    for (int k = 0; k < 2; ++k) {
+      rsd.r[k] = r64v[k];
+      rsd.r32[k] = fp32 ? r32v[k] : nullptr;
+      rsd.p[k] = h->p64[k];
+      rsd.p32[k] = h->p32[k];
     }
+    for (int d = 0; d < 3; ++d) rsd.s[d] = op.s[d];
+    rsd.cmass = op.cmass;
+    rsd.project = singular;
+    rsd.st = st;
+    rsd.rtol = rtol;
+    rsd.delta = fp32 ? delta : 0.0;
+    rsd.maxit = h->maxit;
+    int rc = resid(1);
+    h->st_host[sid].iter = 0;
+    if (rc == SDG_OK) rc = resident_sync(h, sid, s);
+    if (rc != SDG_OK) return rc;
+    floor_res = h->st_host[sid].red[0];
+    a64 += h->st_host[sid].red[1] != 0.0 ? 2 : 1;
+  } else {
+    if (singular) SDG_CK(cudaMemcpyAsync(h->x0buf, x, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    // start: r = b - A x0 (x32 = 0)
+    if (fp32) SDG_CK(cudaMemsetAsync(h->x32, 0, n * sizeof(float), s));
+    SDG_K(apply_plain<double>(h, op, x, h->Ap64, s, 1));
+    ++a64;
+    SDG_K(rel_residual(b, h->Ap64, h->r64, n, st, pa, rtol, h->maxit, fp32 ? delta : 0.0, 1, singular, unscaled, s));
+    if (singular) {
+      int nl = 0;
+      SDG_CK(kernel_restore(h, h->r64, nullptr, s, &nl));
+      h->launches += nl;
+      SDG_K(rel_renorm(h->r64, n, st, pa, 1, s));
+    }
+    SDG_CK(cudaMemcpyAsync(h->st_host + sid, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
+    SDG_CK(cudaStreamSynchronize(s));
+    // the reachable tolerance: three times the FP64 residual floor near x0
+    if (!h->st_host[sid].done) {
+      const int rc = floor_residual(h, op, x, h->st_host[sid].bnorm2, singular, s, &floor_res);
+      if (rc != SDG_OK) return rc;
+      ++a64;
+      if (3.0 * floor_res > rtol) {
+        SolverState& hs = h->st_host[sid];
+        const double tol = 3.0 * floor_res;
+        hs.tol2 = tol * tol * hs.bnorm2 * hs.sigma * hs.sigma;
+        if (hs.rr <= hs.tol2) hs.done = 1;
+        SDG_CK(cudaMemcpyAsync(st, h->st_host + sid, sizeof(SolverState), cudaMemcpyHostToDevice, s));
+      }
+    }
+    if (fp32) SDG_K(rel_convert(h->r64, h->r32, n, st, s));
+    h->st_host[sid].iter = 0;
   }
-  if (fp32) SDG_K(rel_convert(h->r64, h->r32, n, st, s));
-  h->st_host[sid].iter = 0;
   int status = SDG_OK;
   // FP32 iterations: the replacement factor adapts to the segment lengths.
   // A replacement costs an FP64 operator application (about ten FP32
@@ -356,14 +434,23 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   // it returns toward the configured value where they run long.
   constexpr int kMinSeg = 64;
   double delta_cur = delta;
+  double delta2 = fp32 ? delta * delta : 0.0;
   int it_last = 0;
   bool stalled = false;  // FP32 iterations stopped improving above the tolerance
   double eval_res = 0.0;  // rounding of A x itself (computed when the residual stalls)
   double best = -1.0;   // best true residual so far
   int stagnant = 0;     // consecutive replacements without a 1.25x improvement of it
+  auto log_update = [&](int k) {
+    const SolverState& v = h->st_host[sid];
+    if (h->verbose)
+      std::fprintf(stderr, "sdg: reliable update %d at %s iteration %d: true ||r||/||b|| = %.3e\n", k,
+                   fp32 ? "FP32" : "FP64", v.iter, std::sqrt(v.rr) / (v.sigma * std::sqrt(v.bnorm2)));
+  };
   for (;;) {
-    SDG_CK(cudaMemcpyAsync(h->st_host + sid, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
-    SDG_CK(cudaStreamSynchronize(s));
+    if (!whole) {
+      SDG_CK(cudaMemcpyAsync(h->st_host + sid, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
+      SDG_CK(cudaStreamSynchronize(s));
+    }
     if (h->st_host[sid].done) break;
     {
       // a true residual that has stopped improving long before reaching the
@@ -393,8 +480,11 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
       else if (seg > 4 * kMinSeg) d = std::min(std::sqrt(d), delta);
       if (d != delta_cur) {
         delta_cur = d;
-        h->st_host[sid].delta2 = d * d;
-        SDG_CK(cudaMemcpyAsync(&st->delta2, &h->st_host[sid].delta2, sizeof(double), cudaMemcpyHostToDevice, s));
+        delta2 = d * d;
+        if (!resident) {
+          h->st_host[sid].delta2 = d * d;
+          SDG_CK(cudaMemcpyAsync(&st->delta2, &h->st_host[sid].delta2, sizeof(double), cudaMemcpyHostToDevice, s));
+        }
       }
     }
     it_last = h->st_host[sid].iter;
@@ -405,9 +495,30 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
     const long long it_now = h->st_host[sid].iter;
     // (FP64: a segment may at most double the iteration count, FP32: 1/8)
     const long long cap = !fp32 ? (it_now > 5000 ? it_now : 5000) : (it_now / 8 > 2000 ? it_now / 8 : 2000);
-    int rc = fp32 ? cg_loop<float>(h, op, h->x32, r32v, h->p32, Ap32v, sid, s, fused, deflate, cap)
-                  : cg_loop<double>(h, op, x, r64v, h->p64, Ap64v, sid, s, fused, false, cap);
+    int rc;
+    if (resident) {
+      rc = fp32 ? cg_resident<float>(h, op, plan, h->x32, r32v, h->p32, Ap32v, sid, s, cap, delta2)
+                : cg_resident<double>(h, op, plan, x, r64v, h->p64, Ap64v, sid, s, cap, delta2);
+      if (rc == SDG_OK && !whole) rc = resident_sync(h, sid, s);
+    } else
+      rc = fp32 ? cg_loop<float>(h, op, h->x32, r32v, h->p32, Ap32v, sid, s, fused, deflate, cap)
+                : cg_loop<double>(h, op, x, r64v, h->p64, Ap64v, sid, s, fused, false, cap);
     if (rc != SDG_OK) return rc;
+    if (whole) {
+      // residual replacement behind the segment, one round trip for both
+      rc = resid(0);
+      if (rc == SDG_OK) rc = resident_sync(h, sid, s);
+      if (rc != SDG_OK) return rc;
+      ++a64;
+      ++updates;
+      log_update(updates);
+      const SolverState& f = h->st_host[sid];
+      if (f.seg_done || updates >= h->max_updates) {
+        status = f.rr <= f.tol2 ? SDG_OK : (f.seg_done ? f.seg_status : SDG_ERR_NOT_CONVERGED);
+        break;
+      }
+      continue;
+    }
     const SolverState hs = h->st_host[sid];
     // replace the residual (also after a cap or a breakdown, so that x and
     // the reported residual are current): the current residual buffer is
@@ -440,9 +551,7 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
     if (h->verbose) {
       SDG_CK(cudaMemcpyAsync(h->st_host + sid, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
       SDG_CK(cudaStreamSynchronize(s));
-      const SolverState& v = h->st_host[sid];
-      std::fprintf(stderr, "sdg: reliable update %d at %s iteration %d: true ||r||/||b|| = %.3e\n", updates,
-                   fp32 ? "FP32" : "FP64", v.iter, std::sqrt(v.rr) / (v.sigma * std::sqrt(v.bnorm2)));
+      log_update(updates);
     }
     if (hs.done || updates >= h->max_updates) {
       // the iteration hit maxit or broke down, or the update cap is
@@ -459,7 +568,7 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   // CG in exact arithmetic never changes the kernel component of x (every
   // update lies in the range of the operator); rounding does, so put it back
   // to that of x0 (Sec. 2.1: P is defined up to weak solutions of grad p = 0)
-  if (singular) {
+  if (singular && !(whole && h->st_host[sid].restored)) {
     int nl = 0;
     SDG_CK(kernel_restore(h, x, h->x0buf, s, &nl));
     h->launches += nl;
@@ -654,6 +763,14 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
   A_(h->kproj, h->g.n1 * h->g.n1);
   A_(h->kdpart, (size_t)kDeflateBlocks * h->g.npe);
   A_(h->kc, h->g.npe);
+  // resident CG: words of the exchange (FP64 plans: two per published value)
+  const size_t slot_words = (size_t)2 * kResMaxCtas * (8 + 32);  // sums of the iterations, of the replacements
+  for (int k = 0; k < 2; ++k) h->res[k] = res_plan(h, k == 1);
+  const size_t halo_words = h->res[0].state == 1 ? (size_t)4 * n : h->res[1].state == 1 ? (size_t)2 * n : 0;
+  if (halo_words > 0) {
+    A_(h->res_slots, slot_words);
+    A_(h->res_halo, halo_words);
+  }
 #undef A_
   if (rc != SDG_OK) { sdg_destroy(h); return rc; }
   if (cudaMallocHost(&h->st_host, kMaxStates * sizeof(SolverState)) != cudaSuccess) {
@@ -701,6 +818,10 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
     if (e == cudaSuccess) e = cudaMemset(h->kc, 0, npe * sizeof(float));
   }
   if (e == cudaSuccess) e = cudaMemset(h->st, 0, kMaxStates * sizeof(SolverState));
+  // no word of a new handle carries a tag that a launch will use
+  if (e == cudaSuccess && halo_words > 0) e = cudaMemset(h->res_slots, 0, slot_words * sizeof(unsigned long long));
+  if (e == cudaSuccess && halo_words > 0) e = cudaMemset(h->res_halo, 0, halo_words * sizeof(unsigned long long));
+  h->res_tag = h->resid_tag = 1;
   for (int d = 0; d < h->dim && e == cudaSuccess; ++d) e = cudaMemset(h->U[d], 0, n * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->P, 0, n * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->p64[0], 0, n * sizeof(double));
@@ -734,6 +855,7 @@ int sdg_destroy(sdg_handle* h) {
   cudaFree(h->st); cudaFree(h->partials); cudaFree(h->mats);
   cudaFree(h->x0buf); cudaFree(h->kpart); cudaFree(h->kcorr); cudaFree(h->kproj);
   cudaFree(h->kbasis); cudaFree(h->kdpart); cudaFree(h->kc); cudaFree(h->adj);
+  cudaFree(h->res_slots); cudaFree(h->res_halo);
   if (h->st_host) cudaFreeHost(h->st_host);
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);

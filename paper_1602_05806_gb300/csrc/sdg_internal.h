@@ -40,6 +40,10 @@ struct SolverState {
   int nop;          // two-launch form: blocks of the last operator launch (their p.Ap totals
                     // wait in the partials for the update launch)
   unsigned int counter;  // last-block ticket counter (reset by the last block)
+  // resident solve (sdg_cgresid.cuh): done / status of the segment that ended
+  // before the replacement, 1 once x has its kernel part back, 1 / sigma
+  int seg_done, seg_status, restored;
+  double inv_sigma;
 };
 
 // Geometry of a field: element-major blocks of n1^dim nodes.
@@ -64,6 +68,20 @@ constexpr int kReduceBlocks = 152 * 8; // grid of the vector / reduction kernels
 enum StateId { kStP64 = 0, kStP32 = 1, kStV64 = 2, kStV32 = 3, kStMisc = 4, kStTrue = 5 };
 
 constexpr int kProfEvents = 64;  // event pairs per CG batch when profiling
+
+// Resident CG (sdg_cgres.cuh): the tile that gives every CTA its share of the
+// grid, chosen once per handle and precision.
+constexpr int kResMaxSmem = 220 * 1024;  // dynamic shared memory of a CTA
+constexpr int kResMaxN1_3d = 6;          // degrees compiled in 3D (2D: all)
+constexpr int kResMaxCtas = 1024;        // slots of the exchange
+struct ResPlan {
+  int state;    // 1 usable, 2 the grid does not fit
+  int ts[3];    // tile extents in elements
+  int nt[3];    // tiles per direction
+  int threads;  // threads per CTA
+  int lpt;      // x-lines per thread
+  size_t smem;  // dynamic shared memory per CTA
+};
 
 }  // namespace sdg
 
@@ -125,6 +143,12 @@ struct sdg_handle {
   float* kdpart;          // deflation partial sums (kDeflateBlocks * npe)
   float* kc;              // deflation correction pattern (npe)
   cudaEvent_t ev0, ev1, ev2, ev3;
+  // resident CG: plan per precision (0 FP64, 1 FP32), exchange slots of the
+  // sums and of the published Ap (null when no plan is usable), next tag
+  sdg::ResPlan res[2];
+  unsigned long long* res_slots;
+  unsigned long long* res_halo;
+  unsigned res_tag, resid_tag;
   // instrumentation
   long long launches;     // kernels launched by this handle
   int profile;            // time every fused CG operator launch with events
@@ -195,6 +219,57 @@ cudaError_t apply_dispatch_2d(const sdg_handle* h, const ApplyArgs<double>& a, c
 cudaError_t apply_dispatch_2d(const sdg_handle* h, const ApplyArgs<float>& a, cudaStream_t s);
 cudaError_t apply_dispatch_3d(const sdg_handle* h, const ApplyArgs<double>& a, cudaStream_t s);
 cudaError_t apply_dispatch_3d(const sdg_handle* h, const ApplyArgs<float>& a, cudaStream_t s);
+
+// ---- resident CG (sdg_cgres_*.cu) -------------------------------------------
+// Up to cap iterations of the one-launch form in one cooperative launch:
+// vectors of iteration j at index j & 1, x without the last step's alpha p
+// (as ApplyArgs with fuse = 2).  The exchanges of the launch carry the tags
+// tag, tag + 1, ...; a wait that gives up leaves status SDG_ERR_CUDA.
+template <typename T>
+struct ResArgs {
+  T* r[2];
+  T* p[2];
+  T* ap[2];
+  T* x;
+  double s[3];
+  double cmass;
+  SolverState* st;
+  unsigned tag;
+  int cap;
+  double delta2;  // replacement factor squared (the state's value is set to it)
+};
+cudaError_t res_dispatch_2d(const sdg_handle* h, const ResPlan& pl, const ResArgs<double>& a, cudaStream_t s);
+cudaError_t res_dispatch_2d(const sdg_handle* h, const ResPlan& pl, const ResArgs<float>& a, cudaStream_t s);
+cudaError_t res_dispatch_3d(const sdg_handle* h, const ResPlan& pl, const ResArgs<double>& a, cudaStream_t s);
+cudaError_t res_dispatch_3d(const sdg_handle* h, const ResPlan& pl, const ResArgs<float>& a, cudaStream_t s);
+// Start (start = 1) or residual replacement of a resident solve in one
+// cooperative launch with the FP64 plan: x += correction (and the step still
+// owed to x when the iteration stopped at maxit), r = b - A x projected onto
+// the range (project), norm, floor (start: st->red[0], red[1] = 1 if
+// computed) and decisions, and the vectors the iterations go on with.  The
+// exchanges carry the tags tag .. tag + 2.
+struct ResidArgs {
+  const double* b;
+  double* x;
+  double* x0;
+  float* x32;
+  // by parity of the iteration count, as in ResArgs (r32: null in FP64 solves)
+  double* r[2];
+  float* r32[2];
+  const double* p[2];
+  const float* p32[2];
+  double s[3];
+  double cmass;
+  int project, start;
+  SolverState* st;
+  unsigned tag;
+  double rtol, delta;
+  int maxit;
+};
+cudaError_t resid_dispatch_2d(const sdg_handle* h, const ResPlan& pl, const ResidArgs& a, cudaStream_t s);
+cudaError_t resid_dispatch_3d(const sdg_handle* h, const ResPlan& pl, const ResidArgs& a, cudaStream_t s);
+// Plan of the resident kernel for the handle's grid (state 2: none fits).
+ResPlan res_plan(const sdg_handle* h, bool fp32);
 
 // ---- vector / step kernels (sdg_kernels.cu) --------------------------------
 // Update launch of a two-launch CG iteration: alpha from the operator
