@@ -324,6 +324,37 @@ cudaError_t pending_x(float* x, const float* p, long long n, SolverState* st, cu
 // removes the kernel component of x (projection onto the range).
 cudaError_t kernel_restore(const sdg_handle* h, double* x, const double* x0, cudaStream_t s, int* launches);
 
+// ---- line-wise stage kernels (sdg_lines_*.cu) -------------------------------
+// out = base + scale (perpendicular weights, if weights) (K a + s (J K J) b)
+// along d, s = 1 (plus) or -1; a, b read from the element sa, sb away along d
+// (a2 set: a, b stand for c1 a + c2 a2, c1 b + c2 b2); st: the sum of the
+// outputs goes to st->red[0].
+struct PairArgs {
+  int d;
+  const double* K;   // n1 x n1, host
+  const double* K2;  // weights: J K J as computed (term by term form)
+  bool plus, weights;
+  const double *a, *b;
+  int sa, sb;
+  const double *a2, *b2;
+  double c1, c2;
+  const double* base;
+  double scale;
+  double* out;
+  SolverState* st;
+  double* partials;
+};
+cudaError_t pair_dispatch_2d(const sdg_handle* h, const PairArgs& a, cudaStream_t s);
+cudaError_t pair_dispatch_3d(const sdg_handle* h, const PairArgs& a, cudaStream_t s);
+struct ConvArgs {
+  const double* const* V0;
+  const double* const* V;
+  double* const* out;
+  double a, b, dt;
+};
+cudaError_t conv_dispatch_2d(const sdg_handle* h, const ConvArgs& a, cudaStream_t s);
+cudaError_t conv_dispatch_3d(const sdg_handle* h, const ConvArgs& a, cudaStream_t s);
+
 // step stages
 cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s);
 cudaError_t k_main_to_dual(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s);

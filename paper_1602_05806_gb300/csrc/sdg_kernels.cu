@@ -461,148 +461,7 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ------------------------------------------------------------------ step stages
-// Per-node kernels: one thread per output node; the 1D matrices are staged
-// in shared memory because the row index varies across the warp.
-struct StepParams {
-  Geo g;
-  double invdx[3];
-};
-
-__device__ __forceinline__ void load_mats(const double* mats, double* s_m, const int* ids, int nid) {
-  for (int k = 0; k < nid; ++k)
-    for (int i = threadIdx.x; i < kMatStride; i += blockDim.x) s_m[k * kMatStride + i] = mats[ids[k] * kMatStride + i];
-  __syncthreads();
-}
-
-// out[e] = M^-1 (M^L in[e-1] + M^R in[e]) along d   (Eq. l2forward)
-// out[e] = M^-1 (M^L in[e] + M^R in[e+1]) along d   (Eq. l2backward)
-template <bool TO_MAIN>
-__global__ void __launch_bounds__(kThreads)
-    k_project(Geo g, int d, const double* __restrict__ in, double* __restrict__ out, const double* mats) {
-  __shared__ double s_m[3 * kMatStride];
-  const int ids[3] = {kML, kMR, kWinv};
-  load_mats(mats, s_m, ids, 3);
-  const double* ML = s_m;
-  const double* MR = s_m + kMatStride;
-  const double* winv = s_m + 2 * kMatStride;
-  const int n1 = g.n1;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < g.ndof;
-       idx += (long long)gridDim.x * blockDim.x) {
-    int e[3], l[3];
-    split_index(g, idx, e, l);
-    const long long ec = elem_of(g, e);
-    const long long en = elem_shift(g, e, d, TO_MAIN ? -1 : +1);
-    const int m = l[d];
-    int l0[3] = {l[0], l[1], l[2]};
-    l0[d] = 0;
-    const int lb = local_of(g, l0), st = lstride(g, d);
-    const double* a = in + (TO_MAIN ? en : ec) * g.npe + lb;  // multiplied by M^L
-    const double* b = in + (TO_MAIN ? ec : en) * g.npe + lb;  // multiplied by M^R
-    double acc = 0.0;
-    for (int q = 0; q < n1; ++q) acc += ML[m * n1 + q] * a[q * st] + MR[m * n1 + q] * b[q * st];
-    out[idx] = acc * winv[m];
-  }
-}
-
-// Trace of field X of element el at xi = side along d, at the face node given
-// by the other local indices (lb = local base with l_d = 0).
-__device__ __forceinline__ double trace(const double* X, long long el, int npe, int lb, int st, int n1,
-                                        const double* phis) {
-  const double* p = X + el * npe + lb;
-  double s = 0.0;
-  for (int q = 0; q < n1; ++q) s += phis[q] * p[q * st];
-  return s;
-}
-
-// out_c = a V0_c + b (V_c + dt L(V)_c), with the collocated Rusanov DG operator
-//   L(q) = - sum_d (1/dx_d) M_d^-1 [phi(1) F^_{e+1/2} - phi(0) F^_{e-1/2} - Dn^T W (q v_d)]
-// F^ = (q^- v^- + q^+ v^+)/2 - s (q^+ - q^-)/2,  s = 2 max(|v_d^-|, |v_d^+|).
-// Applied by lines: one thread per (element, line along d) forms the four
-// traces and two face fluxes of its line once and the n1 outputs of every
-// component.  Directions run as successive launches: the first writes L, the
-// next add to it, the last writes out_c = a V0_c + b (V_c + dt L_c) instead.
-struct ConvLineParams {
-  Geo g;
-  int d, first, last;
-  double invdx;
-  const double* V0[3];
-  const double* V[3];
-  double* L[3];
-  double* out[3];
-  double a, b, dt;
-};
-
-__global__ void __launch_bounds__(kThreads) k_convect_line(ConvLineParams p, const double* mats) {
-  __shared__ double s_m[5 * kMatStride];
-  const int ids[5] = {kW, kWinv, kPhi0, kPhi1, kDn};
-  load_mats(mats, s_m, ids, 5);
-  const double* w = s_m;
-  const double* winv = s_m + kMatStride;
-  const double* phi0 = s_m + 2 * kMatStride;
-  const double* phi1 = s_m + 3 * kMatStride;
-  const double* Dn = s_m + 4 * kMatStride;
-  const Geo& g = p.g;
-  const int n1 = g.n1, dim = g.dim, d = p.d;
-  const int lpe = g.npe / n1;  // lines per element along d
-  const long long nlines = g.ncell * (long long)lpe;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nlines;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long el = t / lpe;
-    const int lam = (int)(t - el * lpe);
-    int e[3];
-    e[0] = (int)(el % g.n[0]);
-    const long long rest = el / g.n[0];
-    e[1] = (int)(rest % g.n[1]);
-    e[2] = (int)(rest / g.n[1]);
-    if (dim == 2) e[2] = 0;
-    // the other local indices of the line, in increasing direction order
-    int l0[3] = {0, 0, 0};
-    {
-      int r = lam;
-      for (int d2 = 0; d2 < dim; ++d2) {
-        if (d2 == d) continue;
-        l0[d2] = r % n1;
-        r /= n1;
-      }
-    }
-    const int lb = local_of(g, l0), st = lstride(g, d);
-    const long long ec = elem_of(g, e);
-    const long long em = elem_shift(g, e, d, -1), ep = elem_shift(g, e, d, +1);
-    const double* Vd = p.V[d];
-    const double vd_l_m = trace(Vd, em, g.npe, lb, st, n1, phi1);
-    const double vd_l_p = trace(Vd, ec, g.npe, lb, st, n1, phi0);
-    const double vd_r_m = trace(Vd, ec, g.npe, lb, st, n1, phi1);
-    const double vd_r_p = trace(Vd, ep, g.npe, lb, st, n1, phi0);
-    const double s_l = 2.0 * fmax(fabs(vd_l_m), fabs(vd_l_p));
-    const double s_r = 2.0 * fmax(fabs(vd_r_m), fabs(vd_r_p));
-    const double* vdc = Vd + ec * g.npe + lb;
-    for (int c = 0; c < dim; ++c) {
-      const double* Q = p.V[c];
-      const double q_l_m = trace(Q, em, g.npe, lb, st, n1, phi1);
-      const double q_l_p = trace(Q, ec, g.npe, lb, st, n1, phi0);
-      const double q_r_m = trace(Q, ec, g.npe, lb, st, n1, phi1);
-      const double q_r_p = trace(Q, ep, g.npe, lb, st, n1, phi0);
-      const double f_l = 0.5 * (q_l_m * vd_l_m + q_l_p * vd_l_p) - 0.5 * s_l * (q_l_p - q_l_m);
-      const double f_r = 0.5 * (q_r_m * vd_r_m + q_r_p * vd_r_p) - 0.5 * s_r * (q_r_p - q_r_m);
-      const double* qc = Q + ec * g.npe + lb;
-      for (int m = 0; m < n1; ++m) {
-        double vol = 0.0;
-        for (int k = 0; k < n1; ++k) vol += w[k] * Dn[k * n1 + m] * qc[k * st] * vdc[k * st];
-        const double surf = phi1[m] * f_r - phi0[m] * f_l;
-        const long long idx = ec * g.npe + lb + (long long)m * st;
-        const double Lv = (p.first ? 0.0 : p.L[c][idx]) - p.invdx * winv[m] * (surf - vol);
-        if (p.last) {
-          const double v0 = p.a != 0.0 ? p.V0[c][idx] : 0.0;
-          p.out[c][idx] = p.a * v0 + p.b * (Q[idx] + p.dt * Lv);
-        } else {
-          p.L[c][idx] = Lv;
-        }
-      }
-    }
-  }
-}
-
-
+// (the line-wise ones are in sdg_lines.cuh)
 __global__ void __launch_bounds__(kThreads)
     k_mass(Geo g, const double* __restrict__ F, double* __restrict__ b, double* __restrict__ x0,
            const double* mats) {
@@ -621,106 +480,12 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// out = base + scale * sum_d (1/dx_d) M^{perp d} (Rb U_d[e] - Lb U_d[e-1])   (Eq. pSDG1)
-struct DivParams {
-  Geo g;
-  double invdx[3];
-  const double* U[3];
-  const double* base;
-  double scale;
-  double* out;
-};
-
-__global__ void __launch_bounds__(kThreads) k_div(DivParams p, const double* mats, SolverState* st,
-                                                  double* partials) {
-  __shared__ double s_m[3 * kMatStride];
-  const int ids[3] = {kRb, kLb, kW};
-  load_mats(mats, s_m, ids, 3);
-  const double* Rb = s_m;
-  const double* Lb = s_m + kMatStride;
-  const double* w = s_m + 2 * kMatStride;
-  const Geo& g = p.g;
-  const int n1 = g.n1;
-  double sum = 0.0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < g.ndof;
-       idx += (long long)gridDim.x * blockDim.x) {
-    int e[3], l[3];
-    split_index(g, idx, e, l);
-    const long long ec = elem_of(g, e);
-    double acc = 0.0;
-    for (int d = 0; d < g.dim; ++d) {
-      const long long em = elem_shift(g, e, d, -1);
-      const int m = l[d];
-      int l0[3] = {l[0], l[1], l[2]};
-      l0[d] = 0;
-      const int lb = local_of(g, l0), stp = lstride(g, d);
-      const double* uc = p.U[d] + ec * g.npe + lb;
-      const double* um = p.U[d] + em * g.npe + lb;
-      double t = 0.0;
-      for (int q = 0; q < n1; ++q) t += Rb[m * n1 + q] * uc[q * stp] - Lb[m * n1 + q] * um[q * stp];
-      double wp = 1.0;
-      for (int d2 = 0; d2 < g.dim; ++d2)
-        if (d2 != d) wp *= w[l[d2]];
-      acc += p.invdx[d] * wp * t;
-    }
-    const double v = (p.base ? p.base[idx] : 0.0) + p.scale * acc;
-    p.out[idx] = v;
-    sum += v;
-  }
-  double v1[1] = {sum}, tot[1];
-  if (grid_sum<1>(v1, partials, &st->counter, tot) && threadIdx.x == 0) st->red[0] = tot[0];
-}
-
 __global__ void __launch_bounds__(kThreads)
     k_shift_kernel(double* __restrict__ x, long long n, const SolverState* st, int slot, double factor) {
   const double c = st->red[slot] * factor;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     x[i] -= c;
-}
-
-// U_d = U*_d - (dt/dx_d) M^-1 (R~ q[e+1] - L~ q[e]),  q = theta Pn + (1-theta) Po   (Eq. LOvelocityU)
-struct VelParams {
-  Geo g;
-  double coef[3];  // dt / dx_d
-  double theta;
-  const double* Us[3];
-  const double* Pn;
-  const double* Po;
-  double* U[3];
-};
-
-__global__ void __launch_bounds__(kThreads) k_velocity(VelParams p, const double* mats) {
-  __shared__ double s_m[3 * kMatStride];
-  const int ids[3] = {kRt, kLt, kWinv};
-  load_mats(mats, s_m, ids, 3);
-  const double* Rt = s_m;
-  const double* Lt = s_m + kMatStride;
-  const double* winv = s_m + 2 * kMatStride;
-  const Geo& g = p.g;
-  const int n1 = g.n1;
-  const double th = p.theta, th1 = 1.0 - p.theta;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < g.ndof;
-       idx += (long long)gridDim.x * blockDim.x) {
-    int e[3], l[3];
-    split_index(g, idx, e, l);
-    const long long ec = elem_of(g, e);
-    for (int d = 0; d < g.dim; ++d) {
-      const long long ep = elem_shift(g, e, d, +1);
-      const int m = l[d];
-      int l0[3] = {l[0], l[1], l[2]};
-      l0[d] = 0;
-      const int lb = local_of(g, l0), stp = lstride(g, d);
-      double t = 0.0;
-      for (int q = 0; q < n1; ++q) {
-        const long long ic = ec * g.npe + lb + q * stp, ip = ep * g.npe + lb + q * stp;
-        const double qc = th * p.Pn[ic] + th1 * p.Po[ic];
-        const double qp = th * p.Pn[ip] + th1 * p.Po[ip];
-        t += Rt[m * n1 + q] * qp - Lt[m * n1 + q] * qc;
-      }
-      p.U[d][idx] = p.Us[d][idx] - p.coef[d] * winv[m] * t;
-    }
-  }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -924,76 +689,111 @@ cudaError_t rel_convert(const double* r64, float* r32, long long n, const Solver
   return cudaGetLastError();
 }
 
-cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
-  k_project<true><<<grid_full(h->g.ndof), kThreads, 0, s>>>(h->g, d, in, out, h->mats);
-  return cudaGetLastError();
+namespace {
+cudaError_t pair_line(const sdg_handle* h, const PairArgs& a, cudaStream_t s) {
+  return h->dim == 2 ? pair_dispatch_2d(h, a, s) : pair_dispatch_3d(h, a, s);
 }
+// The matrix K of a pair transform K a + s (J K J) b from R and L = J R J,
+// the mean of the two computed ones (each carries the rounding of its own
+// quadrature), rows scaled by 1 / w.
+void pair_matrix(const sdg_handle* h, const double* R, const double* L, double* out) {
+  const int n1 = h->g.n1, last = n1 * n1 - 1;
+  for (int i = 0; i <= last; ++i) out[i] = 0.5 * (R[i] + L[last - i]) / h->basis.w[i / n1];
+}
+}  // namespace
+
+// M^-1 (M^L in[e-1] + M^R in[e]) along d (Eq. l2forward), M^L = J M^R J
+cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
+  double K[kMaxN1 * kMaxN1];
+  pair_matrix(h, h->basis.MR, h->basis.ML, K);
+  PairArgs a{};
+  a.d = d;
+  a.K = K;
+  a.plus = true;
+  a.a = a.b = in;
+  a.sb = -1;
+  a.scale = 1.0;
+  a.out = out;
+  return pair_line(h, a, s);
+}
+// M^-1 (M^L in[e] + M^R in[e+1]) along d (Eq. l2backward)
 cudaError_t k_main_to_dual(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
-  k_project<false><<<grid_full(h->g.ndof), kThreads, 0, s>>>(h->g, d, in, out, h->mats);
-  return cudaGetLastError();
+  double K[kMaxN1 * kMaxN1];
+  pair_matrix(h, h->basis.MR, h->basis.ML, K);
+  PairArgs a{};
+  a.d = d;
+  a.K = K;
+  a.plus = true;
+  a.a = a.b = in;
+  a.sa = 1;
+  a.scale = 1.0;
+  a.out = out;
+  return pair_line(h, a, s);
 }
 cudaError_t k_convect_stage(const sdg_handle* h, const double* const* V0, const double* const* V,
                             double* const* out, double a, double b, double dt, cudaStream_t s) {
-  const long long nlines = h->g.ndof / h->g.n1;
-  for (int d = 0; d < h->dim; ++d) {
-    ConvLineParams q;
-    q.g = h->g;
-    q.d = d;
-    q.first = d == 0;
-    q.last = d == h->dim - 1;
-    q.invdx = 1.0 / h->dx[d];
-    for (int c = 0; c < 3; ++c) {
-      const bool on = c < h->dim;
-      q.V0[c] = on && V0 ? V0[c] : nullptr;
-      q.V[c] = on ? V[c] : nullptr;
-      q.L[c] = on ? h->Lc[c] : nullptr;
-      q.out[c] = on ? out[c] : nullptr;
-    }
-    q.a = a;
-    q.b = b;
-    q.dt = dt;
-    k_convect_line<<<grid_full(nlines), kThreads, 0, s>>>(q, h->mats);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  ConvArgs q{};
+  q.V0 = V0;
+  q.V = V;
+  q.out = out;
+  q.a = a;
+  q.b = b;
+  q.dt = dt;
+  return h->dim == 2 ? conv_dispatch_2d(h, q, s) : conv_dispatch_3d(h, q, s);
 }
 cudaError_t k_mass_rhs(const sdg_handle* h, const double* F, double* b, double* x0, cudaStream_t s) {
   k_mass<<<grid_full(h->g.ndof), kThreads, 0, s>>>(h->g, F, b, x0, h->mats);
   return cudaGetLastError();
 }
+// base + scale sum_d (1/dx_d) M^{perp d} (R-bar U_d[e] - L-bar U_d[e-1]) (Eq. pSDG1), L-bar = J R-bar J;
+// a launch per direction, the last one sums the outputs
 cudaError_t k_divergence(const sdg_handle* h, const double* const* U, const double* base, double scale,
                          double* out, SolverState* st, double* partials, cudaStream_t s) {
-  DivParams p;
-  p.g = h->g;
-  for (int d = 0; d < 3; ++d) {
-    p.invdx[d] = d < h->dim ? 1.0 / h->dx[d] : 0.0;
-    p.U[d] = d < h->dim ? U[d] : nullptr;
+  for (int d = 0; d < h->dim; ++d) {
+    PairArgs a{};
+    a.d = d;
+    a.K = h->basis.Rb;
+    a.K2 = h->basis.Lb;
+    a.weights = true;
+    a.a = a.b = U[d];
+    a.sb = -1;
+    a.base = d == 0 ? base : out;
+    a.scale = scale / h->dx[d];
+    a.out = out;
+    a.st = d == h->dim - 1 ? st : nullptr;
+    a.partials = partials;
+    const cudaError_t e = pair_line(h, a, s);
+    if (e != cudaSuccess) return e;
   }
-  p.base = base;
-  p.scale = scale;
-  p.out = out;
-  k_div<<<grid_for(h->g.ndof), kThreads, 0, s>>>(p, h->mats, st, partials);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 cudaError_t k_shift(double* x, long long n, const SolverState* st, int slot, double factor, cudaStream_t s) {
   k_shift_kernel<<<grid_for(n), kThreads, 0, s>>>(x, n, st, slot, factor);
   return cudaGetLastError();
 }
+// U*_d - (dt/dx_d) M^-1 (R~ q[e+1] - L~ q[e]) (Eq. LOvelocityU), L~ = J R~ J
 cudaError_t k_velocity_update(const sdg_handle* h, const double* const* Ustar, const double* Pn,
                               const double* Po, double* const* U, cudaStream_t s) {
-  VelParams p;
-  p.g = h->g;
-  for (int d = 0; d < 3; ++d) {
-    p.coef[d] = d < h->dim ? h->dt / h->dx[d] : 0.0;
-    p.Us[d] = d < h->dim ? Ustar[d] : nullptr;
-    p.U[d] = d < h->dim ? U[d] : nullptr;
+  double K[kMaxN1 * kMaxN1];
+  pair_matrix(h, h->basis.Rt, h->basis.Lt, K);
+  for (int d = 0; d < h->dim; ++d) {
+    PairArgs a{};
+    a.d = d;
+    a.K = K;
+    a.a = a.b = Pn;
+    a.sa = 1;
+    if (h->theta != 1.0) {  // q = theta Pn + (1 - theta) Po
+      a.a2 = a.b2 = Po;
+      a.c1 = h->theta;
+      a.c2 = 1.0 - h->theta;
+    }
+    a.base = Ustar[d];
+    a.scale = -h->dt / h->dx[d];
+    a.out = U[d];
+    const cudaError_t e = pair_line(h, a, s);
+    if (e != cudaSuccess) return e;
   }
-  p.theta = h->theta;
-  p.Pn = Pn;
-  p.Po = Po;
-  k_velocity<<<grid_full(h->g.ndof), kThreads, 0, s>>>(p, h->mats);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 cudaError_t k_weighted_sum(const sdg_handle* h, const double* x, const double* y, SolverState* st, int slot,
                            double* partials, cudaStream_t s) {
