@@ -238,6 +238,12 @@ int cg_resident(sdg_handle* h, const Op& op, const ResPlan& pl, T* x, T* const* 
   a.tag = h->res_tag;
   a.cap = (int)std::min<long long>(segment_cap, h->maxit);
   a.delta2 = delta2;
+  if constexpr (sizeof(T) == 4) {
+    if (pl.big) {
+      SDG_K(big_dispatch(h, pl, a, s));
+      return SDG_OK;
+    }
+  }
   SDG_K(h->dim == 2 ? res_dispatch_2d(h, pl, a, s) : res_dispatch_3d(h, pl, a, s));
   return SDG_OK;
 }

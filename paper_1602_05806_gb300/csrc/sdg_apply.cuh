@@ -17,6 +17,7 @@
 #pragma once
 
 #include <atomic>
+#include <cstring>
 #include <type_traits>
 
 #include "sdg_device.cuh"
@@ -63,6 +64,19 @@ struct Coef {
   T zn[HO], z2[HO], S0[HO], S1[HO], k1[HO];
   T k0, inv_n;
 };
+
+// The coefficients in both halves of a 64-bit word, for P2 lines.
+template <int N1>
+void dup_coef(const Coef<float, N1>& in, Coef<C2, N1>* out) {
+  static_assert(sizeof(Coef<C2, N1>) == 2 * sizeof(Coef<float, N1>), "same members");
+  const float* f = reinterpret_cast<const float*>(&in);
+  C2* d = reinterpret_cast<C2*>(out);
+  for (size_t i = 0; i < sizeof(in) / sizeof(float); ++i) {
+    unsigned u;
+    std::memcpy(&u, f + i, 4);
+    d[i].v = ((unsigned long long)u << 32) | u;
+  }
+}
 
 template <typename T, int DIM, int N1>
 struct ApplyParams {
@@ -203,8 +217,9 @@ __device__ __forceinline__ void cg_iteration_finish(SolverState* st, double pAp,
 // Eq. pSyst (f: the direction's scale times the perpendicular weight), in
 // the even/odd basis of the line (see Coef), with the accurate contraction
 // when ACC.
-template <typename T, int N1, bool ACC>
-__device__ __forceinline__ void line_apply(const Coef<T, N1>& c, const T (&xl)[N1], const T (&xc)[N1],
+// (T = P2: two lines at once, coefficients C2)
+template <typename T, int N1, bool ACC, typename C = T>
+__device__ __forceinline__ void line_apply(const Coef<C, N1>& c, const T (&xl)[N1], const T (&xc)[N1],
                                            const T (&xr)[N1], T f, T (&val)[N1]) {
   // Even/odd form of the three line segments (see Coef): the neighbour
   // segments enter only through sE = l^_E + r^_E, dE = l^_E - r^_E,

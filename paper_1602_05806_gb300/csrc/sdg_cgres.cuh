@@ -75,6 +75,7 @@ template <>
 struct ResAcc<float> {
   using A = F2;
   static __device__ __forceinline__ A zero() { return F2{0.0f, 0.0f}; }
+  static __device__ __forceinline__ A make(float v) { return F2{v, 0.0f}; }
   static __device__ __forceinline__ A add(A a, A b) { return f2_add(a, b); }
   static __device__ __forceinline__ A shfl(A a, int o) {
     return F2{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
@@ -119,6 +120,7 @@ template <>
 struct ResAcc<double> {
   using A = double;
   static __device__ __forceinline__ A zero() { return 0.0; }
+  static __device__ __forceinline__ A make(double v) { return v; }
   static __device__ __forceinline__ A add(A a, A b) { return a + b; }
   static __device__ __forceinline__ A shfl(A a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
   static __device__ __forceinline__ A from(A a, int l) { return __shfl_sync(0xffffffffu, a, l); }
@@ -158,18 +160,170 @@ __device__ __forceinline__ void res_publish(unsigned long long* base, long long 
   ResAcc<double>::pack(v, w);
   res_store_words(base + 2 * i, w[0], w[1], tag);
 }
-__device__ __forceinline__ bool res_peek(const unsigned long long* base, long long i, unsigned tag, float* v) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(base + i) : "memory");
-  *v = __uint_as_float((unsigned)w);
-  return (unsigned)(w >> 32) == tag;
+// ---- the sums of an iteration ------------------------------------------------
+// p.Ap, r.r, r.Ap, Ap.Ap of a CTA (from its threads' v4) posted in exchange
+// `tag`: lanes halve the four sums between them first.  64 bytes per CTA, so
+// that the store and the readers' loads are whole lines.  All threads call it.
+template <typename T>
+__device__ __forceinline__ void res_post_sums(typename ResAcc<T>::A (&v4)[4], unsigned long long* slot, unsigned tag,
+                                              typename ResAcc<T>::A (*s_red)[4], typename ResAcc<T>::A (*s_tot)[4]) {
+  using TA = ResAcc<T>;
+  using A = typename TA::A;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const bool h16 = lane & 16, h8 = lane & 8;
+  A k0 = h16 ? v4[2] : v4[0], k1 = h16 ? v4[3] : v4[1];
+  A g0 = h16 ? v4[0] : v4[2], g1 = h16 ? v4[1] : v4[3];
+  k0 = TA::add(k0, TA::shfl(g0, 16));
+  k1 = TA::add(k1, TA::shfl(g1, 16));
+  A m0 = h8 ? k1 : k0, m1 = h8 ? k0 : k1;
+  m0 = TA::add(m0, TA::shfl(m1, 8));
+#pragma unroll
+  for (int s = 4; s > 0; s >>= 1) m0 = TA::add(m0, TA::shfl(m0, s));
+  if ((lane & 7) == 0) s_red[wid][(h16 ? 2 : 0) + (h8 ? 1 : 0)] = m0;
+  __syncthreads();
+  if (wid == 0) {
+    const int c4 = lane & 3, w8 = lane >> 2;
+    A t = w8 < nw ? s_red[w8][c4] : TA::zero();
+    if (w8 + 8 < nw) t = TA::add(t, s_red[w8 + 8][c4]);
+#pragma unroll
+    for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
+    if (lane < 4) {
+      if (gridDim.x > 1) {
+        unsigned w[2];
+        TA::pack(t, w);
+        res_store_words(slot + 8 * blockIdx.x + 2 * lane, w[0], w[1], tag);
+      } else {
+        s_tot[0][lane] = t;
+      }
+    }
+  }
 }
-__device__ __forceinline__ bool res_peek(const unsigned long long* base, long long i, unsigned tag, double* v) {
-  unsigned long long a, b;
-  res_load_words(base + 2 * i, a, b);
-  *v = ResAcc<double>::unpack((unsigned)a, (unsigned)b);
-  return (unsigned)(a >> 32) == tag && (unsigned)(b >> 32) == tag;
+
+// polling warps of a CTA: each warp load covers eight CTAs
+__device__ __forceinline__ int res_poll_warps() { return gridDim.x == 1 ? 1 : (blockDim.x >> 5) >= 8 ? 8 : 4; }
+
+// The sums of every CTA, added by the polling warps into s_tot; a lane's loads
+// are in flight together.  False when a wait ran out.
+template <typename T>
+__device__ __forceinline__ bool res_poll_sums(const unsigned long long* slot, unsigned tag,
+                                              typename ResAcc<T>::A (*s_tot)[4]) {
+  using TA = ResAcc<T>;
+  using A = typename TA::A;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int c4 = lane & 3, w8 = lane >> 2, PW = res_poll_warps();
+  bool fail = false;
+  if (wid < PW && gridDim.x > 1) {
+    constexpr int PB = 5;
+    A t = TA::zero();
+    for (int i0 = wid * 8 + w8; i0 < (int)gridDim.x && !fail; i0 += PB * PW * 8) {
+      unsigned long long q0[PB], q1[PB];
+      bool ok;
+      int polls = 0;
+      do {
+        ok = true;
+#pragma unroll
+        for (int u = 0; u < PB; ++u)
+          if (i0 + u * PW * 8 < (int)gridDim.x) res_load_words(slot + 8 * (i0 + u * PW * 8) + 2 * c4, q0[u], q1[u]);
+#pragma unroll
+        for (int u = 0; u < PB; ++u)
+          if (i0 + u * PW * 8 < (int)gridDim.x)
+            ok = ok && (unsigned)(q0[u] >> 32) == tag && (unsigned)(q1[u] >> 32) == tag;
+      } while (!ok && ++polls < kResSpinLimit);
+      fail = !ok;
+      if (ok) {
+#pragma unroll
+        for (int u = 0; u < PB; ++u)
+          if (i0 + u * PW * 8 < (int)gridDim.x) t = TA::add(t, TA::unpack((unsigned)q0[u], (unsigned)q1[u]));
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
+    if (lane < 4) s_tot[wid][lane] = t;
+  }
+  return !fail;
 }
+
+// Warp 0's copy of the recursion, the same in every CTA.
+template <typename T>
+struct ResLoop {
+  using TA = ResAcc<T>;
+  using A = typename TA::A;
+  A alpha, beta, rr, rr_old, pap;
+  T maxrr, tol2, delta2;
+  int it0, it, maxit, cap, done, pause, status;
+  bool reliable;
+  __device__ __forceinline__ void init(const SolverState* st, double d2, int cap_) {
+    alpha = beta = rr = rr_old = pap = TA::zero();
+    maxrr = (T)st->maxrr;
+    tol2 = (T)st->tol2;
+    delta2 = (T)d2;
+    it = it0 = st->iter;
+    maxit = st->maxit;
+    cap = cap_;
+    done = pause = 0;
+    status = st->status;
+    reliable = st->reliable != 0;
+  }
+  // alpha, beta and the decisions (cg_iteration_finish) from the totals, by
+  // warp 0; s_ab and s_flow tell the others
+  __device__ __forceinline__ void decide(A (*s_tot)[4], int fail, T* s_ab, int* s_flow) {
+    const int lane = threadIdx.x & 31, c4 = lane & 3, w8 = lane >> 2;
+    A t = w8 < res_poll_warps() ? s_tot[w8][c4] : TA::zero();
+#pragma unroll
+    for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
+    const A pa = TA::from(t, 0), r2 = TA::from(t, 1), ra = TA::from(t, 2), aa = TA::from(t, 3);
+    const T pa_h = (T)TA::hi(pa), rr_h = (T)TA::hi(r2);
+    pap = pa;
+    rr_old = rr;
+    rr = r2;
+    if (rr_h > maxrr) maxrr = rr_h;
+    if (fail) {
+      done = 1;
+      status = SDG_ERR_CUDA;
+    } else if (!(pa_h > T(0)) || !isfinite(pa_h) || !isfinite(rr_h)) {
+      done = 1;
+      status = SDG_ERR_BREAKDOWN;
+      alpha = TA::zero();
+      beta = TA::zero();
+    } else {
+      // beta = ||r_{k+1}||^2 / ||r_k||^2 = 1 - (2 r.Ap - alpha Ap.Ap) / p.Ap
+      const A iv = TA::inv(pa);
+      alpha = TA::mul(r2, iv);
+      beta = TA::sub(TA::one(), TA::mul(TA::sub(TA::add(ra, ra), TA::mul(alpha, aa)), iv));
+      if (!((T)TA::hi(beta) > T(0))) beta = TA::zero();
+      if (rr_h <= tol2) {
+        if (reliable) pause = 1;
+        else { done = 1; status = SDG_OK; }
+      } else if (reliable && rr_h < delta2 * maxrr) {
+        pause = 1;
+      } else if (it >= maxit) {
+        done = 1;
+        status = SDG_ERR_NOT_CONVERGED;
+      }
+    }
+    if (lane == 0) {
+      s_ab[0] = (T)TA::hi(alpha);
+      s_ab[1] = (T)TA::hi(beta);
+      *s_flow = done || pause || it - it0 >= cap;
+    }
+  }
+  __device__ __forceinline__ void store(SolverState* st, double d2) const {
+    st->pAp = TA::dbl(pap);
+    st->rr_old = it - it0 > 1 ? TA::dbl(rr_old) : st->rr;
+    st->rr = TA::dbl(rr);
+    st->alpha = TA::dbl(alpha);
+    st->beta = TA::dbl(beta);
+    st->alpha_f = (float)TA::hi(alpha);
+    st->beta_f = (float)TA::hi(beta);
+    st->maxrr = (double)maxrr;
+    st->delta2 = d2;
+    st->iter = it;
+    st->done = done;
+    st->pause = pause;
+    st->status = status;
+  }
+};
 
 // ---- tile of a CTA ----------------------------------------------------------
 // Position and extents of the CTA's tile; face halo x-, x+, y-, y+, z-, z+
@@ -303,6 +457,50 @@ __device__ __forceinline__ void res_x_line(const Coef<T, N1>& c, T s0, T cmass, 
   }
 }
 
+// The neighbours' published values of exchange `tag` into s_ah (a halo element
+// after the other), all loads of a thread in flight together; in FP32 two
+// words per load where elements hold an even number of nodes.  False when a
+// wait ran out.
+template <typename T, int NPE>
+__device__ __forceinline__ bool res_fetch(T* s_ah, const int* s_hel, int NH, const unsigned long long* hw, unsigned tag) {
+  constexpr int W = sizeof(T) == 4 && NPE % 2 == 0 ? 2 : 1, HB = 8;
+  constexpr int NV = NPE / W;
+  const int tid = threadIdx.x, nth = blockDim.x, nv = NH * NV;
+  bool fail = false;
+  for (int v0 = tid; v0 < nv && !fail; v0 += HB * nth) {
+    unsigned long long w0[HB], w1[HB];
+    bool ok;
+    int polls = 0;
+    do {
+      ok = true;
+#pragma unroll
+      for (int u = 0; u < HB; ++u) {
+        const int v = v0 + u * nth, s = v / NV;
+        w0[u] = w1[u] = (unsigned long long)tag << 32;
+        if (v >= nv) continue;
+        const unsigned long long* at = hw + (sizeof(T) / 4) * ((size_t)s_hel[s] * NPE + (size_t)((v - s * NV) * W));
+        if constexpr (sizeof(T) == 8 || W == 2) res_load_words(at, w0[u], w1[u]);
+        else asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w0[u]) : "l"(at) : "memory");
+      }
+#pragma unroll
+      for (int u = 0; u < HB; ++u) ok = ok && (unsigned)(w0[u] >> 32) == tag && (unsigned)(w1[u] >> 32) == tag;
+    } while (!ok && ++polls < kResSpinLimit);
+    fail = !ok;
+#pragma unroll
+    for (int u = 0; u < HB; ++u) {
+      const int v = v0 + u * nth;
+      if (v >= nv) continue;
+      if constexpr (sizeof(T) == 8) {
+        s_ah[v] = ResAcc<double>::unpack((unsigned)w0[u], (unsigned)w1[u]);
+      } else {
+        s_ah[v * W] = __uint_as_float((unsigned)w0[u]);
+        if constexpr (W == 2) s_ah[v * W + 1] = __uint_as_float((unsigned)w1[u]);
+      }
+    }
+  }
+  return !fail;
+}
+
 template <typename T, int DIM, int N1, int LPT>
 __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid_constant__ ResParams<T, DIM, N1> a) {
   using TA = ResAcc<T>;
@@ -331,7 +529,7 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
   __shared__ int s_fail;
 
   const int tid = threadIdx.x, nth = blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5, nw = nth >> 5;
+  const int wid = tid >> 5;
   if (tid < N1) s_w[tid] = a.w[tid];
   if (tid == 0) s_fail = 0;
   tile.tables(a.n, a.nt, ES, s_nb, s_hel);
@@ -376,15 +574,10 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
     s_p[(TE + s) * ES + E::node(q)] = fresh ? T(0) : a.p[b0][gi];
   }
 
-  // state of the recursion, the same in every thread of the grid
   T alpha = fresh ? T(0) : (sizeof(T) == 4 ? (T)st->alpha_f : (T)st->alpha);
   T beta = fresh ? T(0) : (sizeof(T) == 4 ? (T)st->beta_f : (T)st->beta);
-  const T tol2 = (T)st->tol2, delta2 = (T)a.delta2;
-  T maxrr = (T)st->maxrr;
-  const bool reliable = st->reliable != 0;
-  const int maxit = st->maxit;
-  A alpha_a = TA::zero(), beta_a = TA::zero(), rr_a = TA::zero(), rr_old = TA::zero(), pap_a = TA::zero();
-  int it = it0, done = 0, pause = 0, status = st->status;
+  ResLoop<T> lp;
+  lp.init(st, a.delta2, a.cap);
 
   for (int k = 0;; ++k) {
     const unsigned tag = a.tag + (unsigned)k;  // of this iteration's exchange
@@ -416,7 +609,8 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
     // ---- Ap: z and y passes into accumulators, x pass in registers ----
     res_cross_passes<T, DIM, N1, LPT>(a.c, a.s, s_w, s_p, s_o, s_nb, TE);
     __syncthreads();
-    T s_pa = T(0), c_pa = T(0), s_rr = T(0), c_rr = T(0), s_ra = T(0), s_aa = T(0);
+    // (sums plain along a line, N1 terms; in FP32 pairs from there on)
+    A v4[4] = {TA::zero(), TA::zero(), TA::zero(), TA::zero()};
 #pragma unroll
     for (int j = 0; j < LPT; ++j) {
       if (!act[j]) continue;
@@ -424,178 +618,33 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
       const int e = id / LINES, lam = id - e * LINES;
       T xc[N1];
       res_x_line<T, DIM, N1>(a.c, a.s[0], a.cmass, s_w, s_p, s_o, s_nb, TE, e, lam, xc, ap[j]);
-#pragma unroll
-      for (int m = 0; m < N1; ++m) {
-        const T v = ap[j][m];
-        // FP32: p.Ap and r.r compensated, r.Ap and Ap.Ap plain (as the
-        // one-launch form); FP64: plain sums of a few terms per thread
-        if constexpr (sizeof(T) == 4) {
-          const T t1 = fma(xc[m], v, -c_pa);
-          const T u1 = s_pa + t1;
-          c_pa = (u1 - s_pa) - t1;
-          s_pa = u1;
-          const T t2 = fma(r[j][m], r[j][m], -c_rr);
-          const T u2 = s_rr + t2;
-          c_rr = (u2 - s_rr) - t2;
-          s_rr = u2;
-        } else {
-          s_pa = fma(xc[m], v, s_pa);
-          s_rr = fma(r[j][m], r[j][m], s_rr);
-        }
-        s_ra = fma(r[j][m], v, s_ra);
-        s_aa = fma(v, v, s_aa);
-      }
       if (pub[j]) {
 #pragma unroll
         for (int m = 0; m < N1; ++m) res_publish(hout, (long long)gl[j] + m, ap[j][m], tag);
       }
-    }
-    // ---- sums of the tile: lanes halve the four sums between them first ----
-    A v4[4];
-    if constexpr (sizeof(T) == 4) {
-      v4[0] = F2{(float)s_pa, -(float)c_pa};
-      v4[1] = F2{(float)s_rr, -(float)c_rr};
-      v4[2] = F2{(float)s_ra, 0.0f};
-      v4[3] = F2{(float)s_aa, 0.0f};
-    } else {
-      v4[0] = s_pa;
-      v4[1] = s_rr;
-      v4[2] = s_ra;
-      v4[3] = s_aa;
-    }
-    {
-      const bool h16 = lane & 16, h8 = lane & 8;
-      A k0 = h16 ? v4[2] : v4[0], k1 = h16 ? v4[3] : v4[1];
-      A g0 = h16 ? v4[0] : v4[2], g1 = h16 ? v4[1] : v4[3];
-      k0 = TA::add(k0, TA::shfl(g0, 16));
-      k1 = TA::add(k1, TA::shfl(g1, 16));
-      A m0 = h8 ? k1 : k0, m1 = h8 ? k0 : k1;
-      m0 = TA::add(m0, TA::shfl(m1, 8));
+      T pa = T(0), rr = T(0), ra = T(0), aa = T(0);
 #pragma unroll
-      for (int s = 4; s > 0; s >>= 1) m0 = TA::add(m0, TA::shfl(m0, s));
-      if ((lane & 7) == 0) s_red[wid][(h16 ? 2 : 0) + (h8 ? 1 : 0)] = m0;
+      for (int m = 0; m < N1; ++m) {
+        pa = fma(xc[m], ap[j][m], pa);
+        rr = fma(r[j][m], r[j][m], rr);
+        ra = fma(r[j][m], ap[j][m], ra);
+        aa = fma(ap[j][m], ap[j][m], aa);
+      }
+      v4[0] = TA::add(v4[0], TA::make(pa));
+      v4[1] = TA::add(v4[1], TA::make(rr));
+      v4[2] = TA::add(v4[2], TA::make(ra));
+      v4[3] = TA::add(v4[3], TA::make(aa));
     }
-    __syncthreads();
-    // ---- the CTA's sums out, everybody's in: 64 bytes per CTA (the four
-    // sums), so that a warp's store and loads are whole lines; PW warps poll
-    // eight CTAs per load, all loads of a lane in flight together ----
-    const int c4 = lane & 3, w8 = lane >> 2;
-    const int PW = gridDim.x == 1 ? 1 : nw >= 8 ? 8 : 4;
     unsigned long long* slot = a.slots + (size_t)(k & 1) * kResMaxCtas * 8;
-    bool fail = false;
-    if (wid == 0) {
-      A t = w8 < nw ? s_red[w8][c4] : TA::zero();
-      if (w8 + 8 < nw) t = TA::add(t, s_red[w8 + 8][c4]);
-#pragma unroll
-      for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
-      if (lane < 4) {
-        if (gridDim.x > 1) {
-          unsigned w[2];
-          TA::pack(t, w);
-          res_store_words(slot + 8 * blockIdx.x + 2 * lane, w[0], w[1], tag);
-        } else {
-          s_tot[0][lane] = t;
-        }
-      }
-    }
-    if (wid < PW && gridDim.x > 1) {
-      constexpr int PB = 5;
-      A t = TA::zero();
-      for (int i0 = wid * 8 + w8; i0 < (int)gridDim.x && !fail; i0 += PB * PW * 8) {
-        unsigned long long q0[PB], q1[PB];
-        bool ok;
-        int polls = 0;
-        do {
-          ok = true;
-#pragma unroll
-          for (int u = 0; u < PB; ++u)
-            if (i0 + u * PW * 8 < (int)gridDim.x) res_load_words(slot + 8 * (i0 + u * PW * 8) + 2 * c4, q0[u], q1[u]);
-#pragma unroll
-          for (int u = 0; u < PB; ++u)
-            if (i0 + u * PW * 8 < (int)gridDim.x)
-              ok = ok && (unsigned)(q0[u] >> 32) == tag && (unsigned)(q1[u] >> 32) == tag;
-        } while (!ok && ++polls < kResSpinLimit);
-        fail = !ok;
-        if (ok) {
-#pragma unroll
-          for (int u = 0; u < PB; ++u)
-            if (i0 + u * PW * 8 < (int)gridDim.x) t = TA::add(t, TA::unpack((unsigned)q0[u], (unsigned)q1[u]));
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
-      if (lane < 4) s_tot[wid][lane] = t;
-    }
-    // the neighbours' Ap for the next update, waited for while other warps
-    // still wait for sums
-    constexpr int HB = 4;
-    for (int v0 = tid; v0 < NH * NPE && !fail; v0 += HB * nth) {
-      long long hg[HB];
-      T hv[HB];
-#pragma unroll
-      for (int u = 0; u < HB; ++u) {
-        const int v = v0 + u * nth, s = v / NPE;
-        hg[u] = v < NH * NPE ? (long long)s_hel[s] * NPE + (v - s * NPE) : -1;
-      }
-      bool ok;
-      int polls = 0;
-      do {
-        ok = true;
-#pragma unroll
-        for (int u = 0; u < HB; ++u)
-          if (hg[u] >= 0) ok = res_peek(hout, hg[u], tag, &hv[u]) && ok;
-      } while (!ok && ++polls < kResSpinLimit);
-      fail = !ok;
-#pragma unroll
-      for (int u = 0; u < HB; ++u)
-        if (hg[u] >= 0) s_ah[v0 + u * nth] = hv[u];
-    }
+    res_post_sums<T>(v4, slot, tag, s_red, s_tot);
+    // the neighbours' Ap for the next update, published before their sums
+    bool fail = NH > 0 && !res_fetch<T, NPE>(s_ah, s_hel, NH, hout, tag);
+    fail = !res_poll_sums<T>(slot, tag, s_tot) || fail;
     if (fail) s_fail = 1;
     __syncthreads();
 
-    // ---- alpha, beta and the decisions (cg_iteration_finish), by one warp ----
-    ++it;
-    if (wid == 0) {
-      A t = w8 < PW ? s_tot[w8][c4] : TA::zero();
-#pragma unroll
-      for (int s = 16; s >= 4; s >>= 1) t = TA::add(t, TA::shfl(t, s));
-      const A pa = TA::from(t, 0), rr = TA::from(t, 1), ra = TA::from(t, 2), aa = TA::from(t, 3);
-      const T pa_h = (T)TA::hi(pa), rr_h = (T)TA::hi(rr);
-      pap_a = pa;
-      rr_old = rr_a;
-      rr_a = rr;
-      if (rr_h > maxrr) maxrr = rr_h;
-      if (s_fail) {
-        done = 1;
-        status = SDG_ERR_CUDA;
-      } else if (!(pa_h > T(0)) || !isfinite(pa_h) || !isfinite(rr_h)) {
-        done = 1;
-        status = SDG_ERR_BREAKDOWN;
-        alpha_a = TA::zero();
-        beta_a = TA::zero();
-      } else {
-        // beta = ||r_{k+1}||^2 / ||r_k||^2 = 1 - (2 r.Ap - alpha Ap.Ap) / p.Ap
-        const A iv = TA::inv(pa);
-        alpha_a = TA::mul(rr, iv);
-        beta_a = TA::sub(TA::one(), TA::mul(TA::sub(TA::add(ra, ra), TA::mul(alpha_a, aa)), iv));
-        if (!((T)TA::hi(beta_a) > T(0))) beta_a = TA::zero();
-        if (rr_h <= tol2) {
-          if (reliable) pause = 1;
-          else { done = 1; status = SDG_OK; }
-        } else if (reliable && rr_h < delta2 * maxrr) {
-          pause = 1;
-        } else if (it >= maxit) {
-          done = 1;
-          status = SDG_ERR_NOT_CONVERGED;
-        }
-      }
-      if (lane == 0) {
-        s_ab[0] = (T)TA::hi(alpha_a);
-        s_ab[1] = (T)TA::hi(beta_a);
-        s_flow = done || pause || it - it0 >= a.cap;
-      }
-    }
+    ++lp.it;
+    if (wid == 0) lp.decide(s_tot, s_fail, s_ab, &s_flow);
     __syncthreads();
     alpha = s_ab[0];
     beta = s_ab[1];
@@ -603,7 +652,7 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
   }
 
   // ---- leave r, p, Ap of the last iteration and x (without its step) ----
-  const int b1 = it & 1;
+  const int b1 = lp.it & 1;
 #pragma unroll
   for (int j = 0; j < LPT; ++j) {
     if (!act[j]) continue;
@@ -618,27 +667,13 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
       a.p[b1][gl[j] + m] = s_p[base + m];
     }
   }
-  if (blockIdx.x == 0 && tid == 0) {
-    st->pAp = TA::dbl(pap_a);
-    st->rr_old = it - it0 > 1 ? TA::dbl(rr_old) : st->rr;
-    st->rr = TA::dbl(rr_a);
-    st->alpha = TA::dbl(alpha_a);
-    st->beta = TA::dbl(beta_a);
-    st->alpha_f = (float)alpha;
-    st->beta_f = (float)beta;
-    st->maxrr = (double)maxrr;
-    st->delta2 = a.delta2;
-    st->iter = it;
-    st->done = done;
-    st->pause = pause;
-    st->status = status;
-  }
+  if (blockIdx.x == 0 && tid == 0) lp.store(st, a.delta2);
 }
 
 // launchers, one per translation unit (sdg_cgres_*.cu)
-template <typename T, int DIM, int N1, int LPT>
-cudaError_t launch_res(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& in, cudaStream_t stream) {
-  ResParams<T, DIM, N1> p;
+template <typename T, int DIM, int N1>
+void fill_res_params(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& in, ResParams<T, DIM, N1>* pp) {
+  ResParams<T, DIM, N1>& p = *pp;
   ApplyParams<T, DIM, N1> q;
   ApplyArgs<T> aa{};
   for (int d = 0; d < 3; ++d) aa.s[d] = in.s[d];
@@ -666,12 +701,18 @@ cudaError_t launch_res(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>&
   p.tag = in.tag;
   p.cap = in.cap;
   p.delta2 = in.delta2;
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(k_cg_res<T, DIM, N1, LPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kResMaxSmem);
+}
+
+// Cooperative launch (all CTAs resident: they wait for one another) of a
+// kernel on the plan's tiles.  The shared-memory attribute is set once per
+// instantiation (twice is harmless: handles of a batch launch from several
+// host threads).
+template <typename P>
+cudaError_t launch_coop(void (*kern)(P), const P& p, const ResPlan& pl, std::atomic<bool>* attr_set, cudaStream_t stream) {
+  if (!attr_set->load(std::memory_order_acquire)) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem);
     if (e != cudaSuccess) return e;
-    attr_set.store(true, std::memory_order_release);
+    attr_set->store(true, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(pl.nt[0] * pl.nt[1] * pl.nt[2]));
@@ -679,13 +720,21 @@ cudaError_t launch_res(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>&
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs resident: they wait for one another
+  attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_cg_res<T, DIM, N1, LPT>, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
+}
+
+template <typename T, int DIM, int N1, int LPT>
+cudaError_t launch_res(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& in, cudaStream_t stream) {
+  ResParams<T, DIM, N1> p;
+  fill_res_params<T, DIM, N1>(h, pl, in, &p);
+  static std::atomic<bool> attr_set{false};
+  return launch_coop(k_cg_res<T, DIM, N1, LPT>, p, pl, &attr_set, stream);
 }
 
 // two x-lines per thread in FP32 where their registers fit (n1 <= 8)

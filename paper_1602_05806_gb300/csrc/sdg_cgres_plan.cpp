@@ -68,6 +68,35 @@ ResPlan res_plan(const sdg_handle* h, bool fp32) {
       }
     }
   }
+  if (best.state == 1 || !fp32 || dim != 2) return best;
+  // larger 2D FP32 tiles: as few rounds of lines per thread as possible, then
+  // the smallest halo
+  const int epr = big_threads(n1) / 32 * (32 / n1);
+  for (int ty = 1; ty <= h->g.n[1]; ++ty) {
+    if (!canonical(1, ty) || nt[1] > most) continue;
+    for (int tx = 1; tx <= h->g.n[0]; ++tx) {
+      const long long te = (long long)ty * tx;
+      if (te > (long long)big_rounds(n1) * epr) break;
+      if (!canonical(0, tx) || (long long)nt[1] * nt[0] > most) continue;
+      const long long nh = (nt[0] > 1 ? 2 * ty : 0) + (nt[1] > 1 ? 2 * tx : 0);
+      const size_t smem = big_smem(n1, te, nh);
+      if (smem > (size_t)kResMaxSmem) continue;
+      const double cost = (double)((te + epr - 1) / epr) * epr + 0.25 * nh;
+      if (best.state == 1 && cost >= best_cost) continue;
+      best_cost = cost;
+      best.state = 1;
+      best.big = 1;
+      best.ts[0] = tx;
+      best.ts[1] = ty;
+      best.ts[2] = 1;
+      best.nt[0] = nt[0];
+      best.nt[1] = nt[1];
+      best.nt[2] = 1;
+      best.lpt = big_rounds(n1);
+      best.threads = big_threads(n1);
+      best.smem = smem;
+    }
+  }
   return best;
 }
 

@@ -417,25 +417,7 @@ cudaError_t launch_resid_t(const sdg_handle* h, const ResPlan& pl, const ResidAr
   p.delta = in.delta;
   p.maxit = in.maxit;
   static std::atomic<bool> attr_set{false};
-  if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_cg_resid<DIM, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem);
-    if (e != cudaSuccess) return e;
-    attr_set.store(true, std::memory_order_release);
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(pl.nt[0] * pl.nt[1] * pl.nt[2]));
-  cfg.blockDim = dim3(pl.threads);
-  cfg.dynamicSmemBytes = pl.smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_cg_resid<DIM, N1>, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_coop(k_cg_resid<DIM, N1>, p, pl, &attr_set, stream);
 }
 
 }  // namespace sdg

@@ -83,6 +83,55 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
   return F2{s, a.lo + b.lo + e};
 }
 
+// ---- two FP32 values per instruction ---------------------------------------
+// A pair of independent floats in one 64-bit register (add / mul / fma.f32x2,
+// each half rounded as the scalar instruction rounds it).  The FP32 rate is
+// that of scalar instructions; a pair takes half their issue slots.
+struct P2 {
+  unsigned long long v;
+  __device__ __forceinline__ P2() {}
+  __device__ __forceinline__ explicit P2(float x) { asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(x)); }
+  __device__ __forceinline__ P2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+  __device__ __forceinline__ float lo() const { return __uint_as_float((unsigned)v); }
+  __device__ __forceinline__ float hi() const { return __uint_as_float((unsigned)(v >> 32)); }
+};
+// The same FP32 coefficient in both halves, as a kernel parameter.
+struct C2 {
+  unsigned long long v;
+};
+using ::fma;
+__device__ __forceinline__ P2 fma(P2 a, P2 b, P2 c) {
+  P2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ P2 fma(float a, P2 b, P2 c) { return fma(P2(a), b, c); }
+__device__ __forceinline__ P2 fma(P2 a, float b, P2 c) { return fma(a, P2(b), c); }
+__device__ __forceinline__ P2 operator+(P2 a, P2 b) {
+  P2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ P2 operator-(P2 a, P2 b) { return fma(P2(-1.0f), b, a); }
+__device__ __forceinline__ P2 operator*(P2 a, P2 b) {
+  P2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ P2 operator*(P2 a, float b) { return a * P2(b); }
+__device__ __forceinline__ P2 as_p2(C2 c) {
+  P2 r;
+  r.v = c.v;
+  return r;
+}
+__device__ __forceinline__ P2 fma(C2 a, P2 b, P2 c) { return fma(as_p2(a), b, c); }
+__device__ __forceinline__ P2 fma(P2 a, C2 b, P2 c) { return fma(a, as_p2(b), c); }
+__device__ __forceinline__ P2 operator*(P2 a, C2 b) { return a * as_p2(b); }
+__device__ __forceinline__ C2 operator-(C2 a) { return C2{a.v ^ 0x8000000080000000ULL}; }
+__device__ __forceinline__ P2 operator-(P2 a) { return a * P2(-1.0f); }
+__device__ __forceinline__ P2& operator+=(P2& a, P2 b) { return a = a + b; }
+__device__ __forceinline__ P2& operator-=(P2& a, P2 b) { return a = a - b; }
+
 // Sum K float pairs over the block; totals (as doubles) in every thread.
 // Warps and then warp 0 add pairs with TwoSum; only the block total is
 // converted to FP64 (one thread).  s_red: at least 32*K doubles.

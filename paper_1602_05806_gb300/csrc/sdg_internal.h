@@ -71,11 +71,24 @@ constexpr int kProfEvents = 64;  // event pairs per CG batch when profiling
 
 // Resident CG (sdg_cgres.cuh): the tile that gives every CTA its share of the
 // grid, chosen once per handle and precision.
-constexpr int kResMaxSmem = 220 * 1024;  // dynamic shared memory of a CTA
+constexpr int kResMaxSmem = 225 * 1024;  // dynamic shared memory of a CTA (the static part stays below 2 KB)
 constexpr int kResMaxN1_3d = 6;          // degrees compiled in 3D (2D: all)
 constexpr int kResMaxCtas = 1024;        // slots of the exchange
+// Large 2D FP32 tiles (sdg_cgbig.cuh), by degree: threads, rounds of lines per
+// thread, rounds whose Ap lives in registers, shared-memory floats per element
+constexpr int big_threads(int) { return 256; }
+constexpr int big_reg_rounds(int) { return 4; }
+constexpr int big_rounds(int n1) { return n1 <= 4 ? 24 : 112 / n1 / 2 * 2; }
+constexpr int big_es(int n1) { return n1 == 8 ? 64 : n1 * (n1 + 1); }  // El2<n1>::ES
+// dynamic shared memory of a tile of te elements with nh halo elements
+constexpr size_t big_smem(int n1, size_t te, size_t nh) {
+  const size_t epr = (size_t)(big_threads(n1) / 32) * (32 / n1), ar = big_reg_rounds(n1);
+  const size_t apn = te > (ar + 2) * epr ? te - ar * epr : 2 * epr;
+  return (te + nh + apn) * big_es(n1) * 4 + te * 16 + nh * 4 + 16;
+}
 struct ResPlan {
   int state;    // 1 usable, 2 the grid does not fit
+  int big;      // 1: the kernel for large tiles
   int ts[3];    // tile extents in elements
   int nt[3];    // tiles per direction
   int threads;  // threads per CTA
@@ -242,6 +255,7 @@ cudaError_t res_dispatch_2d(const sdg_handle* h, const ResPlan& pl, const ResArg
 cudaError_t res_dispatch_2d(const sdg_handle* h, const ResPlan& pl, const ResArgs<float>& a, cudaStream_t s);
 cudaError_t res_dispatch_3d(const sdg_handle* h, const ResPlan& pl, const ResArgs<double>& a, cudaStream_t s);
 cudaError_t res_dispatch_3d(const sdg_handle* h, const ResPlan& pl, const ResArgs<float>& a, cudaStream_t s);
+cudaError_t big_dispatch(const sdg_handle* h, const ResPlan& pl, const ResArgs<float>& a, cudaStream_t s);
 // Start (start = 1) or residual replacement of a resident solve in one
 // cooperative launch with the FP64 plan: x += correction (and the step still
 // owed to x when the iteration stopped at maxit), r = b - A x projected onto

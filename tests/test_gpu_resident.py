@@ -102,3 +102,32 @@ def test_resident_stops_at_maxit(dim, n, N):
         info = h.pressure_cg(dev(np.zeros_like(b)), Z, ok=(sdg.SDG_OK, sdg.SDG_ERR_NOT_CONVERGED))
         assert info["status"] == sdg.SDG_OK and info["iters"] == 0
         assert np.linalg.norm(host(Z) - x0) <= 1e-13 * np.linalg.norm(x0)
+
+
+# grids above one or two lines per thread: large tiles with an odd number of
+# elements, ragged last tiles, one and several rounds past the registers
+LARGE = [((512, 430), 0), ((268, 289), 1), ((300, 290), 2), ((300, 280), 3), ((225, 211), 4), ((119, 257), 5),
+         ((150, 171), 6), ((256, 256), 7), ((160, 150), 7), ((274, 116), 8), ((255, 79), 9), ((110, 120), 10), ((128, 128), 11)]
+
+
+@pytest.mark.parametrize("n,N", LARGE)
+def test_resident_large_tiles(n, N):
+    """Mixed solves on large 2D tiles: the viscous system to 1e-12 and the
+    pressure system to 1e-3, whose FP32 iterations the FP64 residual confirms;
+    residuals evaluated by the oracle (its rounding: below 1e-13)."""
+    L = (TWO_PI, 1.2 * TWO_PI)
+    o = Oracle(Grid(2, n, L), N, 0.05, 0.6, 1e-3)
+    h = sdg.Handle(2, n, L, N, 0.05, 0.6, 1e-3)
+    rng = np.random.default_rng(N)
+    b = o.pressure_apply(rng.standard_normal(o.shape))
+    x0 = rng.standard_normal(o.shape)
+    for A, solve, rtol in ((o.viscous_apply, h.viscous_cg, 1e-12), (o.pressure_apply, h.pressure_cg, 1e-3)):
+        h.set_options(sdg.SDG_MIXED, rtol, rtol, 1000000)
+        before = h.counters()["launches"]
+        X = dev(x0)
+        info = solve(dev(b), X)
+        assert info["status"] == sdg.SDG_OK, info
+        bound = max(rtol, 10.0 * max(info["floor_res"], info["eval_res"]))
+        assert np.linalg.norm(b - A(host(X))) <= (1.01 * bound + 1e-13) * np.linalg.norm(b)
+        # far fewer launches than two per iteration: the resident kernel ran
+        assert info["iters"] < 64 or h.counters()["launches"] - before < info["iters"]
