@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "sdg_internal.h"
@@ -751,35 +752,53 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
   // the operator kernel has one CTA per element box; the smallest box is one
   // element, so ncell bounds every grid (and the reduction grid is capped)
   h->max_blocks = h->g.ncell > kReduceBlocks ? h->g.ncell : kReduceBlocks;
-  int rc = SDG_OK;
-#define A_(p, c) if (rc == SDG_OK) rc = alloc(&(p), (size_t)(c))
-  for (int d = 0; d < h->dim; ++d) {
-    A_(h->U[d], n); A_(h->Vm[d], n); A_(h->S1[d], n); A_(h->S2[d], n);
-    A_(h->F[d], n); A_(h->Vh[d], n); A_(h->Us[d], n); A_(h->Lc[d], n);
-  }
-  A_(h->P, n); A_(h->b, n); A_(h->Pn, n); A_(h->tmp, n);
-  A_(h->r64, n); A_(h->r64b, n); A_(h->p64[0], n); A_(h->p64[1], n); A_(h->Ap64, n); A_(h->Ap64b, n);
-  A_(h->x32, n); A_(h->r32, n); A_(h->r32b, n); A_(h->p32[0], n); A_(h->p32[1], n); A_(h->Ap32, n);
-  A_(h->Ap32b, n);
-  A_(h->st, kMaxStates);
-  A_(h->partials, (size_t)kMaxStates * h->max_blocks * kPartialSlots);
-  A_(h->mats, kMatTable);
-  A_(h->x0buf, n);
-  A_(h->kpart, (size_t)kKernelBlocks * h->g.npe);
-  A_(h->kcorr, h->g.npe);
-  A_(h->kproj, h->g.n1 * h->g.n1);
-  A_(h->kdpart, (size_t)kDeflateBlocks * h->g.npe);
-  A_(h->kc, h->g.npe);
+  // local kernel patterns: tensor products of the 1D basis vectors
+  double b1[kMaxN1 * kMaxN1];
+  const int kd1 = kernel_basis(h->basis, b1);
+  h->kd = 1;
+  for (int d = 0; d < h->dim; ++d) h->kd *= kd1;
   // resident CG: words of the exchange (FP64 plans: two per published value)
   const size_t slot_words = (size_t)2 * kResMaxCtas * (8 + 32);  // sums of the iterations, of the replacements
   for (int k = 0; k < 2; ++k) h->res[k] = res_plan(h, k == 1);
   const size_t halo_words = h->res[0].state == 1 ? (size_t)4 * n : h->res[1].state == 1 ? (size_t)2 * n : 0;
-  if (halo_words > 0) {
-    A_(h->res_slots, slot_words);
-    A_(h->res_halo, halo_words);
+  // one allocation for the fields and workspaces of the handle, measured in a
+  // first pass and handed out in a second, each on a 256-byte boundary (see
+  // sdg_handle::arena)
+  size_t arena_bytes = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    size_t at = 0;
+    auto take = [&](auto*& ptr, size_t count) {
+      if (pass) ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(static_cast<char*>(h->arena) + at);
+      at += (count * sizeof(*ptr) + 255) / 256 * 256;
+    };
+    for (int d = 0; d < h->dim; ++d) {
+      take(h->U[d], n); take(h->Vm[d], n); take(h->S1[d], n); take(h->S2[d], n);
+      take(h->F[d], n); take(h->Vh[d], n); take(h->Us[d], n); take(h->Lc[d], n);
+    }
+    take(h->P, n); take(h->b, n); take(h->Pn, n); take(h->tmp, n);
+    take(h->r64, n); take(h->r64b, n); take(h->p64[0], n); take(h->p64[1], n); take(h->Ap64, n); take(h->Ap64b, n);
+    take(h->x32, n); take(h->r32, n); take(h->r32b, n); take(h->p32[0], n); take(h->p32[1], n); take(h->Ap32, n);
+    take(h->Ap32b, n);
+    take(h->st, kMaxStates);
+    take(h->partials, (size_t)kMaxStates * h->max_blocks * kPartialSlots);
+    take(h->mats, kMatTable);
+    take(h->x0buf, n);
+    take(h->kpart, (size_t)kKernelBlocks * h->g.npe);
+    take(h->kcorr, h->g.npe);
+    take(h->kproj, h->g.n1 * h->g.n1);
+    take(h->kdpart, (size_t)kDeflateBlocks * h->g.npe);
+    take(h->kc, h->g.npe);
+    take(h->kbasis, (size_t)h->kd * h->g.npe);
+    if (halo_words > 0) {
+      take(h->res_slots, slot_words);
+      take(h->res_halo, halo_words);
+    }
+    arena_bytes = at;
+    if (pass == 0) {
+      const int rc = alloc(&h->arena, arena_bytes);
+      if (rc != SDG_OK) { sdg_destroy(h); return rc; }
+    }
   }
-#undef A_
-  if (rc != SDG_OK) { sdg_destroy(h); return rc; }
   if (cudaMallocHost(&h->st_host, kMaxStates * sizeof(SolverState)) != cudaSuccess) {
     sdg_destroy(h);
     set_err("cudaMallocHost failed%s", "");
@@ -801,14 +820,10 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
   for (int k = 0; k < 11; ++k) std::memcpy(table + ids[k] * kMatStride, mats[k], n1 * n1 * sizeof(double));
   cudaError_t e = cudaMemcpy(h->mats, table, sizeof(table), cudaMemcpyHostToDevice);
   {
-    double proj[kMaxN1 * kMaxN1], b1[kMaxN1 * kMaxN1];
+    double proj[kMaxN1 * kMaxN1];
     h->kdim = kernel_projector(h->basis, proj);
     if (e == cudaSuccess) e = cudaMemcpy(h->kproj, proj, n1 * n1 * sizeof(double), cudaMemcpyHostToDevice);
-    // local kernel patterns: tensor products of the 1D basis vectors
-    const int kd1 = kernel_basis(h->basis, b1);
     const int npe = h->g.npe;
-    h->kd = 1;
-    for (int d = 0; d < h->dim; ++d) h->kd *= kd1;
     std::vector<double> kb((size_t)h->kd * npe);
     for (int j = 0; j < h->kd; ++j) {
       int jj = j, idx[3] = {0, 0, 0};
@@ -820,7 +835,6 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
         kb[(size_t)j * npe + l] = v;
       }
     }
-    if (e == cudaSuccess) e = cudaMalloc(&h->kbasis, kb.size() * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpy(h->kbasis, kb.data(), kb.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(h->kc, 0, npe * sizeof(float));
   }
@@ -850,19 +864,8 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
 
 int sdg_destroy(sdg_handle* h) {
   if (!h) return SDG_OK;
-  for (int d = 0; d < 3; ++d) {
-    cudaFree(h->U[d]); cudaFree(h->Vm[d]); cudaFree(h->S1[d]); cudaFree(h->S2[d]);
-    cudaFree(h->F[d]); cudaFree(h->Vh[d]); cudaFree(h->Us[d]); cudaFree(h->Lc[d]);
-  }
-  cudaFree(h->P); cudaFree(h->b); cudaFree(h->Pn); cudaFree(h->tmp);
-  cudaFree(h->r64); cudaFree(h->r64b); cudaFree(h->p64[0]); cudaFree(h->p64[1]); cudaFree(h->Ap64);
-  cudaFree(h->Ap64b);
-  cudaFree(h->x32); cudaFree(h->r32); cudaFree(h->r32b); cudaFree(h->p32[0]); cudaFree(h->p32[1]);
-  cudaFree(h->Ap32); cudaFree(h->Ap32b);
-  cudaFree(h->st); cudaFree(h->partials); cudaFree(h->mats);
-  cudaFree(h->x0buf); cudaFree(h->kpart); cudaFree(h->kcorr); cudaFree(h->kproj);
-  cudaFree(h->kbasis); cudaFree(h->kdpart); cudaFree(h->kc); cudaFree(h->adj);
-  cudaFree(h->res_slots); cudaFree(h->res_halo);
+  cudaFree(h->arena);
+  cudaFree(h->adj);
   if (h->st_host) cudaFreeHost(h->st_host);
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);
