@@ -68,11 +68,15 @@ __host__ __device__ constexpr int m3_halo_slot() {
 }
 
 // Resident CTAs per SM the kernel is compiled for (a register cap: without
-// barriers between the passes the compiler keeps more values live): three
-// in FP32 (48 registers per thread), two in FP64
-template <typename T>
+// barriers between the passes the compiler keeps more values live): three of
+// 400 threads in FP32 for N1 = 5 (48 registers per thread), two in FP64, and
+// what the registers of the passes allow below (N1 = 4: 80 in FP64; with the
+// 88 it would take of itself two CTAs fit, and a CG iteration on 30 x 24 x 27
+// cells took 267 instead of 239 us)
+template <typename T, int N1>
 constexpr int march3_min_blocks() {
-  return sizeof(T) == 4 ? 3 : 2;
+  if (sizeof(T) == 4) return N1 == 5 ? 3 : N1 >= 3 ? 5 : 8;
+  return N1 == 5 ? 2 : N1 == 4 ? 3 : N1 == 3 ? 4 : 8;
 }
 
 // Shared memory of a mode (0 plain apply, 1 operator of the two-launch CG
@@ -101,7 +105,7 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src) {
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <typename T, int N1, bool ACC, int MODE, bool AHEAD>
-__global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T>()))
+__global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T, N1>()))
     k_apply3m(const __grid_constant__ ApplyParams<T, 3, N1> a) {
   using M = March3<N1>;
   using L = March3Smem<T, N1, MODE, AHEAD>;
