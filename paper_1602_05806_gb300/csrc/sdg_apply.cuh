@@ -16,6 +16,7 @@
 // the update launch, which forms alpha (no grid-wide finish here).
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <type_traits>
@@ -63,6 +64,19 @@ struct Coef {
   T rho_e[HE], rho_o[HO];
   T zn[HO], z2[HO], S0[HO], S1[HO], k1[HO];
   T k0, inv_n;
+  // FP64, N1 >= 3: the neighbour blocks by mirror images (see line_apply_fold)
+  static constexpr bool FOLD = std::is_same<T, double>::value && N1 >= 3;
+  T LE[FOLD ? HE * N1 : 1], LO[FOLD ? HO * N1 : 1];
+  void fold() {
+    if constexpr (FOLD) {
+      for (int j = 0; j < N1; ++j) {
+        const int k = j < H ? j : N1 - 1 - j;
+        const T s = j < H ? T(1) : T(-1);
+        for (int m = 0; m < HE; ++m) LE[m * N1 + j] = 2 * j == N1 - 1 ? A[m * HE + H] : A[m * HE + k] - s * B[m * HO + k];
+        for (int m = 0; m < H; ++m) LO[m * N1 + j] = 2 * j == N1 - 1 ? B[H * HO + m] : B[k * HO + m] + s * D[m * HO + k];
+      }
+    }
+  }
 };
 
 // The coefficients in both halves of a 64-bit word, for P2 lines.
@@ -212,6 +226,66 @@ __device__ __forceinline__ void cg_iteration_finish(SolverState* st, double pAp,
   st->beta_f = (float)st->beta;
 }
 
+// line_apply in FP64 for odd N1 (and, without ACC, any N1 >= 3).  H^R = J H^L J
+// (J: reversal of a line), so with a = xl + J xr and b = xl - J xr the
+// neighbours' part of y + J y is a matrix on a and that of y - J y one on b:
+// no even and odd parts of the segments are formed, and of the differences to
+// the centre value only a's, since b's cancel.  Per line of N1 = 5: 74 FP64
+// instructions instead of 91 (ACC), 59 instead of 67; the FP64 pipe bounds
+// every kernel that calls it.  Errors against 128-bit arithmetic over random,
+// smooth, offset and cell-wise constant lines: 0.5 to 1.0 times those of the
+// even/odd form for every N1 >= 3 of these (N1 = 2: up to 1.14, and with the
+// sawtooth's fit of even N1, which a and b see at full size, up to 1.25, so
+// those keep the even/odd form).
+template <int N1, bool ACC>
+__device__ __forceinline__ void line_apply_fold(const Coef<double, N1>& c, const double (&xl)[N1],
+                                                const double (&xc)[N1], const double (&xr)[N1], double f,
+                                                double (&val)[N1]) {
+  constexpr int H = N1 / 2, HE = (N1 + 1) / 2, HO = H > 0 ? H : 1;
+  constexpr bool MID = (N1 % 2) == 1;
+  const double c0 = ACC ? xc[N1 / 2] : 0.0;
+  double a[N1], b[N1], cE[HE], cO[HO];
+#pragma unroll
+  for (int k = 0; k < N1; ++k) {
+    a[k] = ACC ? (xl[k] - c0) + (xr[N1 - 1 - k] - c0) : xl[k] + xr[N1 - 1 - k];
+    b[k] = xl[k] - xr[N1 - 1 - k];
+  }
+#pragma unroll
+  for (int k = 0; k < H; ++k) {
+    cE[k] = ACC ? (xc[k] - c0) + (xc[N1 - 1 - k] - c0) : xc[k] + xc[N1 - 1 - k];
+    cO[k] = xc[k] - xc[N1 - 1 - k];
+  }
+  if constexpr (MID) cE[H] = ACC ? 0.0 : xc[H];
+  double yE[HE], yO[HO];
+#pragma unroll
+  for (int m = 0; m < HE; ++m) {
+    double t = 0.0;
+#pragma unroll
+    for (int j = 0; j < N1; ++j) t = fma(c.LE[m * N1 + j], a[j], t);
+#pragma unroll
+    for (int j = 0; j < (ACC && MID ? H : HE); ++j) t = fma(c.CE[m * HE + j], cE[j], t);
+    if (ACC && m < H) t = fma(-c.rho_e[m], cE[m], t);
+    yE[m] = t;
+  }
+#pragma unroll
+  for (int m = 0; m < H; ++m) {
+    double t = 0.0;
+#pragma unroll
+    for (int j = 0; j < N1; ++j) t = fma(c.LO[m * N1 + j], b[j], t);
+#pragma unroll
+    for (int j = 0; j < H; ++j) t = fma(c.CO[m * HO + j], cO[j], t);
+    if (ACC) t = fma(-c.rho_o[m], cO[m], t);
+    yO[m] = t;
+  }
+#pragma unroll
+  for (int m = 0; m < H; ++m) {
+    const double t = f * yE[m];
+    val[m] = fma(f, yO[m], t);
+    val[N1 - 1 - m] = fma(-f, yO[m], t);
+  }
+  if constexpr (MID) val[H] = f * yE[H];
+}
+
 // The 1D line operator of one direction applied to one line of nodes: the
 // outputs val[m] = f (H^L xl + H^C xc + H^R xr)[m] of the block row of
 // Eq. pSyst (f: the direction's scale times the perpendicular weight), in
@@ -221,6 +295,10 @@ __device__ __forceinline__ void cg_iteration_finish(SolverState* st, double pAp,
 template <typename T, int N1, bool ACC, typename C = T>
 __device__ __forceinline__ void line_apply(const Coef<C, N1>& c, const T (&xl)[N1], const T (&xc)[N1],
                                            const T (&xr)[N1], T f, T (&val)[N1]) {
+  if constexpr (std::is_same<T, double>::value && N1 >= 3 && (!ACC || N1 % 2 == 1)) {
+    line_apply_fold<N1, ACC>(c, xl, xc, xr, f, val);
+    return;
+  }
   // Even/odd form of the three line segments (see Coef): the neighbour
   // segments enter only through sE = l^_E + r^_E, dE = l^_E - r^_E,
   // sO = l^_O + r^_O, dO = r^_O - l^_O, the centre through cE, cO.
@@ -762,6 +840,7 @@ void fill_apply_params(const sdg_handle* h, const ApplyArgs<T>& in, ApplyParams<
   }
   p.c.k0 = (T)cs.k0;
   p.c.inv_n = (T)cs.inv_n;
+  p.c.fold();
   for (int i = 0; i < N1; ++i) p.w[i] = (T)b.w[i];
   p.x = in.x;
   p.p_old = in.p_old;
@@ -792,14 +871,26 @@ cudaError_t launch_apply_acc(const sdg_handle* h, const ApplyArgs<T>& in, cudaSt
   p.ntile[2] = (p.n[2] + TS::TZ - 1) / TS::TZ;
   const long long nblk = (long long)p.ntile[0] * p.ntile[1] * p.ntile[2];
   if (nblk > h->max_blocks) return cudaErrorInvalidConfiguration;
-  const size_t smem = (size_t)(TS::NSLOT + TS::TE) * TS::ES * sizeof(T);
-  // per instantiation (its shared-memory need is fixed); handles of a batch
+  size_t smem = (size_t)(TS::NSLOT + TS::TE) * TS::ES * sizeof(T);
+  size_t smem_max = smem;
+  if constexpr (sizeof(T) == 8) {
+    // An operator launched while the update before it still runs fills the
+    // SMs as their update blocks end, each with as many CTAs as fit: where
+    // the grid is less than a wave, the first SMs get all of it and the FP64
+    // pipes of the others idle.  It asks for so much shared memory that no SM
+    // takes more than its share (100 x 90 cells, N = 6, 299 CTAs of which
+    // four fit: 86 -> 67.5 us per iteration; 180 x 170, N = 2: 68 -> 47).
+    smem_max = std::max(smem, (size_t)kResMaxSmem - 4096);
+    const long long share = (nblk + h->nsm - 1) / h->nsm;
+    if (in.pdl && share <= 8) smem = std::max(smem, (size_t)(kResMaxSmem / share - 4096));
+  }
+  // per instantiation (its largest need is fixed); handles of a batch
   // launch from several host threads, and setting the attribute twice is
   // harmless
   static std::atomic<bool> attr_set{false};
   if (!attr_set.load(std::memory_order_acquire)) {
     cudaError_t e = cudaFuncSetAttribute(k_apply<T, DIM, N1, ACC, V, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         (int)smem_max);
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
