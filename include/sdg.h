@@ -200,11 +200,15 @@ int sdg_set_convection_substeps(sdg_handle* h, int nsub);
  * k-1 (r -= alpha Ap, x += alpha p) while it stages its input, and reduces
  * p.Ap, r.r, r.Ap and Ap.Ap, from which beta is formed one iteration ahead.
  * 1: two launches per iteration, the operator (p = r + beta p, Ap, p.Ap)
- * and the update (x += alpha p, r -= alpha Ap, r.r).  2 (default): two
- * launches, with x += alpha p moved into the next operator launch (which
- * reads p already), so that the update moves only r and Ap.  All are the CG
- * of Sec. 2.1 in exact arithmetic; the FP32 kernel deflation of
- * sdg_set_mixed_options always uses form 1.
+ * and the update (x += alpha p, r -= alpha Ap, r.r).  2 (default): where
+ * one tile of elements per SM holds the grid, one cooperative launch for all
+ * iterations up to the next residual replacement (the recurrence of form 0,
+ * one exchange of sums and face values per iteration); on larger grids, with
+ * profiling on or a tile shape other than 0, two launches, with x += alpha p
+ * moved into the next operator launch (which reads p already), so that the
+ * update moves only r and Ap.  All are the CG of Sec. 2.1 in exact
+ * arithmetic; the FP32 kernel deflation of sdg_set_mixed_options always uses
+ * form 1.
  * Errors: INVALID_ARG unless form is 0, 1 or 2. */
 int sdg_set_iteration_form(sdg_handle* h, int form);
 
@@ -365,7 +369,8 @@ int sdg_batch_step(sdg_batch* b, int nsteps, sdg_step_info* info, void* stream);
 
 /* enable != 0: bracket every launch of the fused CG operator kernel with CUDA
  * events on the launch stream and accumulate its device time (costs a few
- * microseconds of host time per launch).  Resets the counters below. */
+ * microseconds of host time per launch; the default iteration form then runs
+ * its two launches on every grid).  Resets the counters below. */
 int sdg_set_profiling(sdg_handle* h, int enable);
 
 /* Counters since sdg_create or the last sdg_set_profiling: kernels launched
