@@ -53,27 +53,34 @@ struct Tile {
   static constexpr int ES = DIM == 2 ? PS : N1 * PS;
 };
 
+// FP64, N1 >= 3: the neighbour blocks by mirror images (see line_apply_fold)
+template <typename T, int N1, bool F = std::is_same<T, double>::value && (N1 >= 3)>
+struct FoldCoef {};
+template <int N1>
+struct FoldCoef<double, N1, true> {
+  double LE[(N1 + 1) / 2 * N1], LO[N1 / 2 * N1];
+};
+
 // Stored line operator in the compute precision, in the even/odd basis of
 // the line (see CoefSet): H^R = [[A, B], [-B^T, D]], H^L = [[A, -B], [B^T, D]],
 // H^C = diag(CE, CO); kernel correction rho (even N) or the fit and
 // S0 / S1 correction (odd N).
 template <typename T, int N1>
-struct Coef {
+struct Coef : FoldCoef<T, N1> {
   static constexpr int H = N1 / 2, HE = (N1 + 1) / 2, HO = H > 0 ? H : 1;
   T A[HE * HE], B[HE * HO], D[HO * HO], CE[HE * HE], CO[HO * HO];
   T rho_e[HE], rho_o[HO];
   T zn[HO], z2[HO], S0[HO], S1[HO], k1[HO];
   T k0, inv_n;
-  // FP64, N1 >= 3: the neighbour blocks by mirror images (see line_apply_fold)
-  static constexpr bool FOLD = std::is_same<T, double>::value && N1 >= 3;
-  T LE[FOLD ? HE * N1 : 1], LO[FOLD ? HO * N1 : 1];
   void fold() {
-    if constexpr (FOLD) {
+    if constexpr (std::is_same<T, double>::value && N1 >= 3) {
       for (int j = 0; j < N1; ++j) {
         const int k = j < H ? j : N1 - 1 - j;
         const T s = j < H ? T(1) : T(-1);
-        for (int m = 0; m < HE; ++m) LE[m * N1 + j] = 2 * j == N1 - 1 ? A[m * HE + H] : A[m * HE + k] - s * B[m * HO + k];
-        for (int m = 0; m < H; ++m) LO[m * N1 + j] = 2 * j == N1 - 1 ? B[H * HO + m] : B[k * HO + m] + s * D[m * HO + k];
+        for (int m = 0; m < HE; ++m)
+          this->LE[m * N1 + j] = 2 * j == N1 - 1 ? A[m * HE + H] : A[m * HE + k] - s * B[m * HO + k];
+        for (int m = 0; m < H; ++m)
+          this->LO[m * N1 + j] = 2 * j == N1 - 1 ? B[H * HO + m] : B[k * HO + m] + s * D[m * HO + k];
       }
     }
   }
