@@ -212,6 +212,13 @@ int sdg_set_convection_substeps(sdg_handle* h, int nsub);
  * Errors: INVALID_ARG unless form is 0, 1 or 2. */
 int sdg_set_iteration_form(sdg_handle* h, int form);
 
+/* Polls after which a wait of the cooperative CG launches (for the sums and
+ * face values of the other blocks) gives up; 0 (default): 2^22, some seconds.
+ * No wait runs out while the GPU works.  One that does ends the solve with
+ * SDG_ERR_CUDA: x is then undefined, the handle stays usable.
+ * Errors: INVALID_ARG unless polls >= 0. */
+int sdg_set_wait_limit(sdg_handle* h, int polls);
+
 /* Tile shape of the operator kernel.  2D FP32 (a CTA's box of elements):
  * 0 = base, 1 = twice as wide in x, 2 = twice as wide in y (fewer halo
  * loads per element, twice the threads per CTA).  3D: 0 = columns of 4 x 4

@@ -219,10 +219,23 @@ int cg_loop(sdg_handle* h, const Op& op, T* x, T* const* r, T* const* p, T* cons
   return SDG_OK;
 }
 
+// The first of `need` tags no word of the exchange carries.  Tags are used
+// once; before they would run out, the words are cleared (behind the launches
+// that read them) and the tags start again.
+int take_tags(sdg_handle* h, unsigned* next, unsigned need, cudaStream_t s, unsigned* tag) {
+  if (*next > 0xffffffffu - need) {
+    SDG_CK(cudaMemsetAsync(h->res_slots, 0, h->res_words * sizeof(unsigned long long), s));
+    h->res_tag = h->resid_tag = 1;
+  }
+  *tag = *next;
+  *next += need;
+  return SDG_OK;
+}
+
 // Iterations of one segment in the resident kernel: until the device pauses or
 // stops the solve, or segment_cap iterations.  Buffers and x as in the
-// one-launch form of cg_loop.  The caller reads the state back and advances
-// the tag by the iterations done plus one (resident_sync).
+// one-launch form of cg_loop.  The caller reads the state back
+// (resident_sync).
 template <typename T>
 int cg_resident(sdg_handle* h, const Op& op, const ResPlan& pl, T* x, T* const* r, T* const* p, T* const* Ap, int sid,
                 cudaStream_t s, long long segment_cap, double delta2) {
@@ -236,9 +249,11 @@ int cg_resident(sdg_handle* h, const Op& op, const ResPlan& pl, T* x, T* const* 
   for (int d = 0; d < 3; ++d) a.s[d] = op.s[d];
   a.cmass = op.cmass;
   a.st = st_dev(h, sid);
-  a.tag = h->res_tag;
   a.cap = (int)std::min<long long>(segment_cap, h->maxit);
   a.delta2 = delta2;
+  const int rc = take_tags(h, &h->res_tag, (unsigned)a.cap + 1u, s, &a.tag);
+  if (rc != SDG_OK) return rc;
+  h->res_seg = a.tag;
   if constexpr (sizeof(T) == 4) {
     if (pl.big) {
       SDG_K(big_dispatch(h, pl, a, s));
@@ -254,10 +269,15 @@ int resident_sync(sdg_handle* h, int sid, cudaStream_t s) {
   const int it0 = h->st_host[sid].iter;
   SDG_CK(cudaMemcpyAsync(h->st_host + sid, st_dev(h, sid), sizeof(SolverState), cudaMemcpyDeviceToHost, s));
   SDG_CK(cudaStreamSynchronize(s));
-  h->res_tag += (unsigned)(h->st_host[sid].iter - it0) + 1u;
-  if (h->st_host[sid].status == SDG_ERR_CUDA) {
+  if (h->st_host[sid].wait_failed) {  // the tags stay those of a segment that ran to its cap
+    h->res_seg = 0;
+    SDG_CK(cudaMemsetAsync(&st_dev(h, sid)->wait_failed, 0, sizeof(int), s));
     set_err("a wait of the resident CG kernel ran out%s", "");
     return SDG_ERR_CUDA;
+  }
+  if (h->res_seg != 0) {
+    h->res_tag = h->res_seg + (unsigned)(h->st_host[sid].iter - it0) + 1u;
+    h->res_seg = 0;
   }
   return SDG_OK;
 }
@@ -368,12 +388,13 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   float* r32v[2] = {h->r32, fused ? h->r32b : h->r32};
   float* Ap32v[2] = {h->Ap32, fused ? h->Ap32b : h->Ap32};
   int a64 = 0, updates = 0;
+  h->res_seg = 0;  // (not 0 after a solve that ended with an error: its tags stay taken)
   double floor_res = 0.0;
   ResidArgs rsd{};  // start and replacements of a whole resident solve
   auto resid = [&](int start) -> int {
     rsd.start = start;
-    rsd.tag = h->resid_tag;
-    h->resid_tag += 3u;
+    const int rc = take_tags(h, &h->resid_tag, 3u, s, &rsd.tag);
+    if (rc != SDG_OK) return rc;
     SDG_K(h->dim == 2 ? resid_dispatch_2d(h, h->res[0], rsd, s) : resid_dispatch_3d(h, h->res[0], rsd, s));
     return SDG_OK;
   };
@@ -739,6 +760,7 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
   h->form = 2;  // measured faster than the other forms (2D and 3D)
   h->maxit = 1000000;
   h->max_updates = 10000;
+  h->polls = kResPolls;
   build_basis(N, &h->basis);
   build_coefs(h->basis, 0, &h->coef64);
   build_coefs(h->basis, 1, &h->coef32);
@@ -789,9 +811,10 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
     take(h->kdpart, (size_t)kDeflateBlocks * h->g.npe);
     take(h->kc, h->g.npe);
     take(h->kbasis, (size_t)h->kd * h->g.npe);
-    if (halo_words > 0) {
-      take(h->res_slots, slot_words);
-      take(h->res_halo, halo_words);
+    if (halo_words > 0) {  // (one run of words: slots, then halo)
+      h->res_words = slot_words + halo_words;
+      take(h->res_slots, h->res_words);
+      if (pass) h->res_halo = h->res_slots + slot_words;
     }
     arena_bytes = at;
     if (pass == 0) {
@@ -840,8 +863,7 @@ int sdg_create(const sdg_grid* grid, int N, double nu, double theta, double dt, 
   }
   if (e == cudaSuccess) e = cudaMemset(h->st, 0, kMaxStates * sizeof(SolverState));
   // no word of a new handle carries a tag that a launch will use
-  if (e == cudaSuccess && halo_words > 0) e = cudaMemset(h->res_slots, 0, slot_words * sizeof(unsigned long long));
-  if (e == cudaSuccess && halo_words > 0) e = cudaMemset(h->res_halo, 0, halo_words * sizeof(unsigned long long));
+  if (e == cudaSuccess && halo_words > 0) e = cudaMemset(h->res_slots, 0, h->res_words * sizeof(unsigned long long));
   h->res_tag = h->resid_tag = 1;
   for (int d = 0; d < h->dim && e == cudaSuccess; ++d) e = cudaMemset(h->U[d], 0, n * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->P, 0, n * sizeof(double));
@@ -910,6 +932,13 @@ int sdg_set_iteration_form(sdg_handle* h, int form) {
   SDG_ARG(h, "NULL handle");
   SDG_ARG(form >= 0 && form <= 2, "iteration form must be 0, 1 or 2");
   h->form = form;
+  return SDG_OK;
+}
+
+int sdg_set_wait_limit(sdg_handle* h, int polls) {
+  SDG_ARG(h, "NULL handle");
+  SDG_ARG(polls >= 0, "polls must be >= 0");
+  h->polls = polls > 0 ? polls : kResPolls;
   return SDG_OK;
 }
 

@@ -46,7 +46,7 @@ __device__ __forceinline__ void big_publish2(unsigned long long* w, float a, flo
 // a thread in flight together (by fours they took 9800 of 70000 cycles).
 template <int N1>
 __device__ __forceinline__ bool big_fetch_halo(float* s_p, const int* s_hel, int TE, int NH,
-                                               const unsigned long long* hw, unsigned tag) {
+                                               const unsigned long long* hw, unsigned tag, int limit) {
   using B = BigEl<N1>;
   constexpr int NPE = N1 * N1, NT = B::NT, W = NPE % 2 == 0 ? 2 : 1, HB = 12;
   const int nv = NH * (NPE / W);
@@ -68,7 +68,7 @@ __device__ __forceinline__ bool big_fetch_halo(float* s_p, const int* s_hel, int
       }
 #pragma unroll
       for (int u = 0; u < HB; ++u) ok = ok && (unsigned)(w0[u] >> 32) == tag && (unsigned)(w1[u] >> 32) == tag;
-    } while (!ok && ++polls < kResSpinLimit);
+    } while (!ok && ++polls < limit);
     fail = !ok;
 #pragma unroll
     for (int u = 0; u < HB; ++u) {
@@ -311,12 +311,11 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
       }
     }
     __syncthreads();
-    bool fail = false;
     // the last turn of the loop below before one that reads the halo
     const bool early = NI < 2 * EPR;
     const int jf = early ? -1 : (NI / (2 * EPR) - 1) * 2;
     if (NH > 0 && early) {
-      fail = !big_fetch_halo<N1>(s_p, s_hel, TE, NH, hw, tag);
+      if (!big_fetch_halo<N1>(s_p, s_hel, TE, NH, hw, tag, a.polls)) s_fail = st->wait_failed = 1;
       __syncthreads();
     }
 
@@ -384,7 +383,7 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
       }
       __syncwarp();  // the next rounds may use the same places
       if (j == jf && NH > 0) {
-        fail = !big_fetch_halo<N1>(s_p, s_hel, TE, NH, hw, tag);
+        if (!big_fetch_halo<N1>(s_p, s_hel, TE, NH, hw, tag, a.polls)) s_fail = st->wait_failed = 1;
         __syncthreads();
       }
     }
@@ -392,9 +391,12 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
     // ---- sums, alpha, beta, decisions ----
     F2 v4[4] = {s_pa, s_rr, s_ra, s_aa};
     unsigned long long* slot = a.slots + (size_t)(k & 1) * kResMaxCtas * 8;
-    if (fail) s_fail = 1;
-    res_post_sums<float>(v4, slot, tag, s_red, s_tot);
-    if (!res_poll_sums<float>(slot, tag, s_tot)) s_fail = 1;
+    // (sums formed with an old halo are not posted; s_fail is the same for all
+    // threads here, the fetch being behind a barrier)
+    if (!s_fail) {
+      res_post_sums<float>(v4, slot, tag, s_red, s_tot);
+      if (!res_poll_sums<float>(slot, tag, a.polls, s_tot)) s_fail = st->wait_failed = 1;
+    }
     __syncthreads();
     if (wid == 0) {
       ResLoop<float> lp = s_lp;

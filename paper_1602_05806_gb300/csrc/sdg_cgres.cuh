@@ -22,8 +22,9 @@
 // of a line delay its writers, so few whole lines are best.)  Two parities of
 // words alternate: a CTA writes exchange k + 2 only after every CTA has
 // written k + 1, that is, has read all it needs of k.  Waits are bounded: a
-// reader that gives up sets the state's status and leaves, and so does every
-// CTA that waits for it.
+// CTA that gives up sets the state's wait_failed and leaves without posting
+// anything more, and so does every CTA that waits for it; the host reports
+// SDG_ERR_CUDA.
 //
 // A CTA keeps its copy of the neighbours' r and p on its face halo and
 // advances it with the published Ap (the same arithmetic as the owner's), so
@@ -38,8 +39,6 @@
 #include "sdg_apply.cuh"
 
 namespace sdg {
-
-constexpr int kResSpinLimit = 1 << 22; // polls before a wait gives up (seconds)
 
 // threads per CTA the kernel is compiled for: 255 registers in FP64, 128 in FP32
 template <typename T>
@@ -65,6 +64,7 @@ struct ResParams {
   long long ndof;
   unsigned tag;               // exchange k of this launch carries tag + k
   int cap;                    // most iterations of this launch
+  int polls;                  // of a wait before it gives up
   double delta2;              // pause when r.r < delta2 (its largest value so far)
 };
 
@@ -205,7 +205,7 @@ __device__ __forceinline__ int res_poll_warps() { return gridDim.x == 1 ? 1 : (b
 // The sums of every CTA, added by the polling warps into s_tot; a lane's loads
 // are in flight together.  False when a wait ran out.
 template <typename T>
-__device__ __forceinline__ bool res_poll_sums(const unsigned long long* slot, unsigned tag,
+__device__ __forceinline__ bool res_poll_sums(const unsigned long long* slot, unsigned tag, int limit,
                                               typename ResAcc<T>::A (*s_tot)[4]) {
   using TA = ResAcc<T>;
   using A = typename TA::A;
@@ -228,7 +228,7 @@ __device__ __forceinline__ bool res_poll_sums(const unsigned long long* slot, un
         for (int u = 0; u < PB; ++u)
           if (i0 + u * PW * 8 < (int)gridDim.x)
             ok = ok && (unsigned)(q0[u] >> 32) == tag && (unsigned)(q1[u] >> 32) == tag;
-      } while (!ok && ++polls < kResSpinLimit);
+      } while (!ok && ++polls < limit);
       fail = !ok;
       if (ok) {
 #pragma unroll
@@ -462,7 +462,8 @@ __device__ __forceinline__ void res_x_line(const Coef<T, N1>& c, T s0, T cmass, 
 // words per load where elements hold an even number of nodes.  False when a
 // wait ran out.
 template <typename T, int NPE>
-__device__ __forceinline__ bool res_fetch(T* s_ah, const int* s_hel, int NH, const unsigned long long* hw, unsigned tag) {
+__device__ __forceinline__ bool res_fetch(T* s_ah, const int* s_hel, int NH, const unsigned long long* hw, unsigned tag,
+                                          int limit) {
   constexpr int W = sizeof(T) == 4 && NPE % 2 == 0 ? 2 : 1, HB = 8;
   constexpr int NV = NPE / W;
   const int tid = threadIdx.x, nth = blockDim.x, nv = NH * NV;
@@ -484,7 +485,7 @@ __device__ __forceinline__ bool res_fetch(T* s_ah, const int* s_hel, int NH, con
       }
 #pragma unroll
       for (int u = 0; u < HB; ++u) ok = ok && (unsigned)(w0[u] >> 32) == tag && (unsigned)(w1[u] >> 32) == tag;
-    } while (!ok && ++polls < kResSpinLimit);
+    } while (!ok && ++polls < limit);
     fail = !ok;
 #pragma unroll
     for (int u = 0; u < HB; ++u) {
@@ -638,9 +639,9 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
     unsigned long long* slot = a.slots + (size_t)(k & 1) * kResMaxCtas * 8;
     res_post_sums<T>(v4, slot, tag, s_red, s_tot);
     // the neighbours' Ap for the next update, published before their sums
-    bool fail = NH > 0 && !res_fetch<T, NPE>(s_ah, s_hel, NH, hout, tag);
-    fail = !res_poll_sums<T>(slot, tag, s_tot) || fail;
-    if (fail) s_fail = 1;
+    bool fail = NH > 0 && !res_fetch<T, NPE>(s_ah, s_hel, NH, hout, tag, a.polls);
+    fail = !res_poll_sums<T>(slot, tag, a.polls, s_tot) || fail;
+    if (fail) s_fail = st->wait_failed = 1;
     __syncthreads();
 
     ++lp.it;
@@ -700,6 +701,7 @@ void fill_res_params(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& i
   p.ndof = h->g.ndof;
   p.tag = in.tag;
   p.cap = in.cap;
+  p.polls = h->polls;
   p.delta2 = in.delta2;
 }
 

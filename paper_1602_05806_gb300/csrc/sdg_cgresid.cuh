@@ -40,6 +40,7 @@ struct ResidParams {
   SolverState* st;
   unsigned long long* slots;  // [2 parities][kResMaxCtas][16 sums][2 words]
   unsigned tag;
+  int polls;            // of a wait before it gives up
   int start;            // 1: start of a solve
   double rtol, delta;
   int maxit;
@@ -47,9 +48,9 @@ struct ResidParams {
 
 // The sums v[0..15] of every thread of the grid, in s_sum of every CTA.
 // Exchange number `tag`, parity `par`.  All threads of the block call it;
-// false when a wait ran out.
-__device__ __forceinline__ void resid_exchange(double (&v)[16], unsigned long long* slots, unsigned tag, int par,
-                                               double (*s_red)[16], double* s_sum, int* s_fail) {
+// false (for all of them) when a wait of the CTA ran out: it leaves then.
+__device__ __forceinline__ bool resid_exchange(double (&v)[16], unsigned long long* slots, unsigned tag, int par,
+                                               int limit, double (*s_red)[16], double* s_sum, int* s_fail) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
   // lanes halve the values between them: lane pair 2 i, 2 i + 1 ends with value i
 #pragma unroll
@@ -98,7 +99,7 @@ __device__ __forceinline__ void resid_exchange(double (&v)[16], unsigned long lo
         for (int u = 0; u < PB; ++u)
           if (i0 + u * nw * 2 < (int)gridDim.x)
             ok = ok && (unsigned)(q0[u] >> 32) == tag && (unsigned)(q1[u] >> 32) == tag;
-      } while (!ok && ++polls < kResSpinLimit);
+      } while (!ok && ++polls < limit);
       if (ok) {
 #pragma unroll
         for (int u = 0; u < PB; ++u)
@@ -117,6 +118,7 @@ __device__ __forceinline__ void resid_exchange(double (&v)[16], unsigned long lo
     }
   }
   __syncthreads();
+  return *s_fail == 0;
 }
 
 // 2^floor(log2 |x|) / (2^52 2 sqrt 3) with the sign of an integer hash of the
@@ -244,7 +246,11 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
       }
     }
   }
-  resid_exchange(v, a.slots, a.tag, 0, s_red, s_sum, &s_fail);
+  // a CTA whose wait ran out posts nothing more and writes no vector
+  auto give_up = [&] {
+    if (tid == 0) st->wait_failed = 1;
+  };
+  if (!resid_exchange(v, a.slots, a.tag, 0, a.polls, s_red, s_sum, &s_fail)) return give_up();
   const double ndof = a.ncell * (double)NPE;
   const double bb = s_sum[2], uu0 = s_sum[4], us = s_sum[3];
   double ss = s_sum[1];
@@ -264,7 +270,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
     for (int i = 0; i < 16; ++i) v[i] = 0.0;
 #pragma unroll
     for (int m = 0; m < N1; ++m) v[0] = fma(r[m], r[m], v[0]);
-    resid_exchange(v, a.slots, a.tag + 1, 1, s_red, s_sum, &s_fail);
+    if (!resid_exchange(v, a.slots, a.tag + 1, 1, a.polls, s_red, s_sum, &s_fail)) return give_up();
     ss = s_sum[0];
   }
 
@@ -289,10 +295,6 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
     if (!isfinite(rr)) {
       done = 1;
       status = SDG_ERR_BREAKDOWN;
-    }
-    if (s_fail) {
-      done = 1;
-      status = SDG_ERR_CUDA;
     }
     if (tid == 0) {
       s_dd[0] = sg;
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
           if (j < a.kd) v[5 + j] = fma(s_kb[j * NPE + lam * N1 + m], d, v[5 + j]);
       }
     }
-    resid_exchange(v, a.slots, a.tag + 2, 0, s_red, s_sum, &s_fail);
+    if (!resid_exchange(v, a.slots, a.tag + 2, 0, a.polls, s_red, s_sum, &s_fail)) return give_up();
     if (act) {
 #pragma unroll
       for (int j = 0; j < kResidMaxKd; ++j) {
@@ -412,6 +414,7 @@ cudaError_t launch_resid_t(const sdg_handle* h, const ResPlan& pl, const ResidAr
   p.st = in.st;
   p.slots = h->res_slots + (size_t)2 * kResMaxCtas * 8;
   p.tag = in.tag;
+  p.polls = h->polls;
   p.start = in.start;
   p.rtol = in.rtol;
   p.delta = in.delta;

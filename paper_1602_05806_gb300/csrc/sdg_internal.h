@@ -44,6 +44,9 @@ struct SolverState {
   // before the replacement, 1 once x has its kernel part back, 1 / sigma
   int seg_done, seg_status, restored;
   double inv_sigma;
+  // set by any CTA of a resident launch whose wait ran out; cleared by the
+  // host once it has reported it
+  int wait_failed;
 };
 
 // Geometry of a field: element-major blocks of n1^dim nodes.
@@ -74,6 +77,7 @@ constexpr int kProfEvents = 64;  // event pairs per CG batch when profiling
 constexpr int kResMaxSmem = 225 * 1024;  // dynamic shared memory of a CTA (the static part stays below 2 KB)
 constexpr int kResMaxN1_3d = 6;          // degrees compiled in 3D (2D: all)
 constexpr int kResMaxCtas = 1024;        // slots of the exchange
+constexpr int kResPolls = 1 << 22;       // polls before a wait gives up (seconds), see sdg_set_wait_limit
 // Large 2D FP32 tiles (sdg_cgbig.cuh), by degree: threads, rounds of lines per
 // thread, rounds whose Ap lives in registers, shared-memory floats per element
 constexpr int big_threads(int) { return 256; }
@@ -162,11 +166,16 @@ struct sdg_handle {
   float* kc;              // deflation correction pattern (npe)
   cudaEvent_t ev0, ev1, ev2, ev3;
   // resident CG: plan per precision (0 FP64, 1 FP32), exchange slots of the
-  // sums and of the published Ap (null when no plan is usable), next tag
+  // sums and of the published Ap (null when no plan is usable; res_words of
+  // both in all), next tags (the iterations' res_tag as if every segment ran
+  // to its cap, until resident_sync has read how far the one from res_seg on
+  // got), polls of a wait
   sdg::ResPlan res[2];
   unsigned long long* res_slots;
   unsigned long long* res_halo;
-  unsigned res_tag, resid_tag;
+  size_t res_words;
+  unsigned res_tag, res_seg, resid_tag;
+  int polls;
   // instrumentation
   long long launches;     // kernels launched by this handle
   int profile;            // time every fused CG operator launch with events
@@ -242,7 +251,7 @@ cudaError_t apply_dispatch_3d(const sdg_handle* h, const ApplyArgs<float>& a, cu
 // Up to cap iterations of the one-launch form in one cooperative launch:
 // vectors of iteration j at index j & 1, x without the last step's alpha p
 // (as ApplyArgs with fuse = 2).  The exchanges of the launch carry the tags
-// tag, tag + 1, ...; a wait that gives up leaves status SDG_ERR_CUDA.
+// tag, tag + 1, ...; a wait that gives up sets the state's wait_failed.
 template <typename T>
 struct ResArgs {
   T* r[2];

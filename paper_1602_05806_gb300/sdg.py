@@ -27,7 +27,7 @@ SDG_MIXED = 1
 # every symbol include/sdg.h declares
 EXPORTS = (
     "sdg_nodes", "sdg_matrices", "sdg_kernel_projector", "sdg_line_operator", "sdg_create", "sdg_destroy", "sdg_set_options",
-    "sdg_set_mixed_options", "sdg_set_convection_substeps", "sdg_set_iteration_form", "sdg_set_tile", "sdg_autotune", "sdg_ndof", "sdg_set_state", "sdg_get_state",
+    "sdg_set_mixed_options", "sdg_set_convection_substeps", "sdg_set_iteration_form", "sdg_set_wait_limit", "sdg_set_tile", "sdg_autotune", "sdg_ndof", "sdg_set_state", "sdg_get_state",
     "sdg_pressure_apply", "sdg_viscous_apply", "sdg_pressure_cg", "sdg_viscous_cg",
     "sdg_dual_to_main", "sdg_main_to_dual", "sdg_convect", "sdg_pressure_rhs",
     "sdg_velocity_update", "sdg_step", "sdg_step_adjoint", "sdg_set_profiling", "sdg_counters", "sdg_diagnostics",
@@ -85,6 +85,7 @@ def lib():
         L.sdg_set_convection_substeps.argtypes = [vp, ip]
         L.sdg_set_tile.argtypes = [vp, ip]
         L.sdg_set_iteration_form.argtypes = [vp, ip]
+        L.sdg_set_wait_limit.argtypes = [vp, ip]
         L.sdg_autotune.argtypes = [vp, ctypes.POINTER(ctypes.c_int), dp, vp]
         L.sdg_ndof.argtypes = [vp]
         L.sdg_ndof.restype = ctypes.c_longlong
@@ -254,6 +255,10 @@ class Handle:
         """0: one launch per CG iteration; 1: operator + update launches, x += alpha p in the update;
         2 (default): operator + update launches, x += alpha p in the next operator launch."""
         check(lib().sdg_set_iteration_form(self.h, int(form)))
+
+    def set_wait_limit(self, polls=0):
+        """Polls after which a wait between the blocks of a cooperative CG launch gives up (0: the default)."""
+        check(lib().sdg_set_wait_limit(self.h, int(polls)))
 
     def set_tile(self, variant):
         """Tile shape of the 2D FP32 operator (0 base, 1 wide in x, 2 wide in y)."""
