@@ -204,9 +204,9 @@ int sdg_set_convection_substeps(sdg_handle* h, int nsub);
  * one tile of elements per SM holds the grid, one cooperative launch for all
  * iterations up to the next residual replacement (the recurrence of form 0,
  * one exchange of sums and face values per iteration); on larger grids, with
- * profiling on or a tile shape other than 0, two launches, with x += alpha p
- * moved into the next operator launch (which reads p already), so that the
- * update moves only r and Ap.  All are the CG of Sec. 2.1 in exact
+ * profiling on or an operator shape asked for (sdg_set_tile), two launches,
+ * with x += alpha p moved into the next operator launch (which reads p
+ * already), so that the update moves only r and Ap.  All are the CG of Sec. 2.1 in exact
  * arithmetic; the FP32 kernel deflation of sdg_set_mixed_options always uses
  * form 1.
  * Errors: INVALID_ARG unless form is 0, 1 or 2. */
@@ -227,12 +227,17 @@ int sdg_set_wait_limit(sdg_handle* h, int polls);
  * shape changes the summation order of the CG's dot products, so results
  * differ in the last bits between shapes (each is deterministic).  The
  * one-launch CG iteration (sdg_set_iteration_form) uses the base 2D shape.
+ * A shape other than 0 keeps solves of its precision (2D: FP32 iterations,
+ * 3D: both) on the two-launch form, which launches that operator, on grids
+ * where the default form would otherwise run cooperative launches.
  * Errors: INVALID_ARG. */
 int sdg_set_tile(sdg_handle* h, int variant);
 /* Times the FP32 operator of the handle's grid with every tile shape (10
  * launches each, CUDA events on `stream`), keeps the fastest and returns it
  * in *variant (may be NULL); us (may be NULL) receives the mean launch time
- * of each shape in microseconds (3 entries in 2D, 2 in 3D).  No counterpart
+ * of each shape in microseconds (3 entries in 2D, 2 in 3D).  The shape found
+ * serves the operator wherever it is launched; unlike sdg_set_tile it does not
+ * move a solve from cooperative launches to that operator.  No counterpart
  * in the paper: a tuning aid.  Synchronises the stream. */
 int sdg_autotune(sdg_handle* h, int* variant, double* us, void* stream);
 

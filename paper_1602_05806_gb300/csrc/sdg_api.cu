@@ -375,10 +375,11 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   const int unscaled = fp32 ? 0 : 1;
   // the default form on grids whose tiles fit the GPU at once: the resident
   // kernel, which runs the one-launch form's iteration (with every launch to
-  // be timed, or a tile shape asked for, the iterations stay single launches);
-  // its replacements are one launch too where the FP64 tiles fit (whole)
+  // be timed, or an operator shape asked for that this precision has, the
+  // iterations stay single launches); its replacements are one launch too
+  // where the FP64 tiles fit (whole)
   const ResPlan& plan = h->res[fp32 ? 1 : 0];
-  const bool resident = !deflate && h->form == 2 && h->tile32 == 0 && !h->profile && plan.state == 1;
+  const bool resident = !deflate && h->form == 2 && !(h->tile_asked && (fp32 || h->dim == 3)) && !h->profile && plan.state == 1;
   const bool whole = resident && h->res[0].state == 1;
   // one launch per iteration or less unless asked otherwise or the FP32
   // iteration deflates the kernel
@@ -946,6 +947,7 @@ int sdg_set_tile(sdg_handle* h, int variant) {
   SDG_ARG(h, "NULL handle");
   SDG_ARG(variant >= 0 && variant <= 2, "tile variant must be 0, 1 or 2");
   h->tile32 = h->dim == 2 ? variant : (variant ? 1 : 0);
+  h->tile_asked = h->tile32 != 0;
   return SDG_OK;
 }
 
@@ -974,6 +976,7 @@ int sdg_autotune(sdg_handle* h, int* variant, double* us, void* stream) {
     }
   }
   h->tile32 = pick;
+  h->tile_asked = 0;
   if (variant) *variant = pick;
   return SDG_OK;
 }

@@ -111,6 +111,7 @@ struct sdg_handle {
   double nu, theta, dt;
   int nsub;                      // SSP-RK3 sub-steps of the explicit convection per dt
   int tile32;                    // tile shape variant of the 2D FP32 operator
+  int tile_asked;                // 1: asked for by sdg_set_tile (0: the base shape, or what sdg_autotune found)
   int form;                      // CG iteration form: 0 one launch, 1 / 2 operator + update launches
   int precision;
   double rtol_p, rtol_v;
