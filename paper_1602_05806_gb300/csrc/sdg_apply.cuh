@@ -17,7 +17,6 @@
 #pragma once
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <type_traits>
 
@@ -891,15 +890,13 @@ cudaError_t launch_apply_acc(const sdg_handle* h, const ApplyArgs<T>& in, cudaSt
     const long long share = (nblk + h->nsm - 1) / h->nsm;
     if (in.pdl && share <= 8) smem = std::max(smem, (size_t)(kResMaxSmem / share - 4096));
   }
-  // per instantiation (its largest need is fixed); handles of a batch
-  // launch from several host threads, and setting the attribute twice is
-  // harmless
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set.load(std::memory_order_acquire)) {
+  // per instantiation (its largest need is fixed) and device
+  static PerDevice attr_set;
+  if (!attr_set.get(h->device)) {
     cudaError_t e = cudaFuncSetAttribute(k_apply<T, DIM, N1, ACC, V, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem_max);
     if (e != cudaSuccess) return e;
-    attr_set.store(true, std::memory_order_release);
+    attr_set.set(h->device, 1);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)nblk);

@@ -641,20 +641,21 @@ cudaError_t launch_apply3m(const sdg_handle* h, const ApplyArgs<T>& in, cudaStre
   fill_apply_params<T, 3, N1>(h, in, &p);
   const size_t smem = (size_t)March3Smem<T, N1, MODE, AHEAD>::SZ * sizeof(T);
   // resident CTAs per SM of this instantiation (fixed: threads and shared
-  // memory do not depend on the grid), measured once
-  static std::atomic<int> occ{0};
-  if (occ.load(std::memory_order_acquire) == 0) {
+  // memory do not depend on the grid), asked once per device
+  static PerDevice occ_of;
+  int occ = occ_of.get(h->device);
+  if (occ == 0) {
     cudaError_t e = cudaFuncSetAttribute(k_apply3m<T, N1, ACC, MODE, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    int o = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_apply3m<T, N1, ACC, MODE, AHEAD>, M::THREADS, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply3m<T, N1, ACC, MODE, AHEAD>, M::THREADS, smem);
     if (e != cudaSuccess) return e;
-    occ.store(o > 0 ? o : 1, std::memory_order_release);
+    if (occ < 1) occ = 1;
+    occ_of.set(h->device, occ);
   }
   p.ntile[0] = (p.n[0] + M::TX - 1) / M::TX;
   p.ntile[1] = (p.n[1] + M::TY - 1) / M::TY;
-  p.zc = march3_zc(p.ntile[0], p.ntile[1], p.n[2], (long long)h->nsm * occ.load(std::memory_order_acquire));
+  p.zc = march3_zc(p.ntile[0], p.ntile[1], p.n[2], (long long)h->nsm * occ);
   p.ntile[2] = (p.n[2] + p.zc - 1) / p.zc;
   const long long nblk = (long long)p.ntile[0] * p.ntile[1] * p.ntile[2];
   if (nblk > h->max_blocks) return cudaErrorInvalidConfiguration;

@@ -436,8 +436,8 @@ cudaError_t launch_big(const sdg_handle* h, const ResPlan& pl, const ResArgs<flo
   BigParams<N1> p;
   fill_res_params<float, 2, N1>(h, pl, in, &p);
   dup_coef(p.c, &p.c2);
-  static std::atomic<bool> attr_set{false};
-  return launch_coop(k_cg_big<N1>, p, pl, &attr_set, stream);
+  static PerDevice attr_set;
+  return launch_coop(k_cg_big<N1>, p, h, pl, &attr_set, stream);
 }
 
 }  // namespace sdg

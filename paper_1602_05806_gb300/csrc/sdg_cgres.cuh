@@ -707,14 +707,14 @@ void fill_res_params(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& i
 
 // Cooperative launch (all CTAs resident: they wait for one another) of a
 // kernel on the plan's tiles.  The shared-memory attribute is set once per
-// instantiation (twice is harmless: handles of a batch launch from several
-// host threads).
+// instantiation and device.
 template <typename P>
-cudaError_t launch_coop(void (*kern)(P), const P& p, const ResPlan& pl, std::atomic<bool>* attr_set, cudaStream_t stream) {
-  if (!attr_set->load(std::memory_order_acquire)) {
+cudaError_t launch_coop(void (*kern)(P), const P& p, const sdg_handle* h, const ResPlan& pl, PerDevice* attr_set,
+                        cudaStream_t stream) {
+  if (!attr_set->get(h->device)) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem);
     if (e != cudaSuccess) return e;
-    attr_set->store(true, std::memory_order_release);
+    attr_set->set(h->device, 1);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(pl.nt[0] * pl.nt[1] * pl.nt[2]));
@@ -735,8 +735,8 @@ template <typename T, int DIM, int N1, int LPT>
 cudaError_t launch_res(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& in, cudaStream_t stream) {
   ResParams<T, DIM, N1> p;
   fill_res_params<T, DIM, N1>(h, pl, in, &p);
-  static std::atomic<bool> attr_set{false};
-  return launch_coop(k_cg_res<T, DIM, N1, LPT>, p, pl, &attr_set, stream);
+  static PerDevice attr_set;
+  return launch_coop(k_cg_res<T, DIM, N1, LPT>, p, h, pl, &attr_set, stream);
 }
 
 // two x-lines per thread in FP32 where their registers fit (n1 <= 8)

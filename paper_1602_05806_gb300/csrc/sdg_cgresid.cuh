@@ -419,8 +419,8 @@ cudaError_t launch_resid_t(const sdg_handle* h, const ResPlan& pl, const ResidAr
   p.rtol = in.rtol;
   p.delta = in.delta;
   p.maxit = in.maxit;
-  static std::atomic<bool> attr_set{false};
-  return launch_coop(k_cg_resid<DIM, N1>, p, pl, &attr_set, stream);
+  static PerDevice attr_set;
+  return launch_coop(k_cg_resid<DIM, N1>, p, h, pl, &attr_set, stream);
 }
 
 }  // namespace sdg

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 
@@ -90,6 +91,20 @@ constexpr size_t big_smem(int n1, size_t te, size_t nh) {
   const size_t apn = te > (ar + 2) * epr ? te - ar * epr : 2 * epr;
   return (te + nh + apn) * big_es(n1) * 4 + te * 16 + nh * 4 + 16;
 }
+// What a launcher keeps of its kernel for every device (function attributes
+// hold for one device only): 0 until it is set.  Handles of a batch launch
+// from several host threads; setting it twice is harmless.
+struct PerDevice {
+  static constexpr int kDevices = 64;  // beyond these nothing is kept
+  std::atomic<int> v[kDevices] = {};
+  int get(int device) const {
+    return device < kDevices ? v[device].load(std::memory_order_acquire) : 0;
+  }
+  void set(int device, int value) {
+    if (device < kDevices) v[device].store(value, std::memory_order_release);
+  }
+};
+
 struct ResPlan {
   int state;    // 1 usable, 2 the grid does not fit
   int big;      // 1: the kernel for large tiles
