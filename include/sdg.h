@@ -204,11 +204,12 @@ int sdg_set_convection_substeps(sdg_handle* h, int nsub);
  * one tile of elements per SM holds the grid, one cooperative launch for all
  * iterations up to the next residual replacement (the recurrence of form 0,
  * one exchange of sums and face values per iteration); on larger grids, with
- * profiling on or an operator shape asked for (sdg_set_tile), two launches,
- * with x += alpha p moved into the next operator launch (which reads p
- * already), so that the update moves only r and Ap.  All are the CG of Sec. 2.1 in exact
- * arithmetic; the FP32 kernel deflation of sdg_set_mixed_options always uses
- * form 1.
+ * profiling on, with an operator shape asked for (sdg_set_tile) or where the
+ * GPU refuses the cooperative launch (fewer SMs for the stream's context than
+ * the device has), two launches, with x += alpha p moved into the next operator
+ * launch (which reads p already), so that the update moves only r and Ap.  All
+ * are the CG of Sec. 2.1 in exact arithmetic; the FP32 kernel deflation of
+ * sdg_set_mixed_options always uses form 1.
  * Errors: INVALID_ARG unless form is 0, 1 or 2. */
 int sdg_set_iteration_form(sdg_handle* h, int form);
 

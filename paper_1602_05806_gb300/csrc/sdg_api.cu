@@ -219,6 +219,19 @@ int cg_loop(sdg_handle* h, const Op& op, T* x, T* const* r, T* const* p, T* cons
   return SDG_OK;
 }
 
+// Internal status of a cooperative launch that the GPU refuses because the
+// stream's context has fewer SMs than the plan counts on.
+constexpr int kRefused = -1;
+
+int cooperative_launch(sdg_handle* h, cudaError_t e) {
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    return kRefused;
+  }
+  SDG_K(e);
+  return SDG_OK;
+}
+
 // The first of `need` tags no word of the exchange carries.  Tags are used
 // once; before they would run out, the words are cleared (behind the launches
 // that read them) and the tags start again.
@@ -255,13 +268,9 @@ int cg_resident(sdg_handle* h, const Op& op, const ResPlan& pl, T* x, T* const* 
   if (rc != SDG_OK) return rc;
   h->res_seg = a.tag;
   if constexpr (sizeof(T) == 4) {
-    if (pl.big) {
-      SDG_K(big_dispatch(h, pl, a, s));
-      return SDG_OK;
-    }
+    if (pl.big) return cooperative_launch(h, big_dispatch(h, pl, a, s));
   }
-  SDG_K(h->dim == 2 ? res_dispatch_2d(h, pl, a, s) : res_dispatch_3d(h, pl, a, s));
-  return SDG_OK;
+  return cooperative_launch(h, h->dim == 2 ? res_dispatch_2d(h, pl, a, s) : res_dispatch_3d(h, pl, a, s));
 }
 
 // The state after a resident segment (and what was launched behind it).
@@ -364,7 +373,8 @@ int eval_residual(sdg_handle* h, const Op& op, const double* x, double bnorm2, c
 // operator (its kernel part is round-off of b and of A x, which no iteration
 // can reduce and which, left in, ends near-kernel directions in breakdown).
 int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, double rtol, int sid,
-                   sdg_cg_info* info, cudaStream_t s, bool singular, bool fp32, int sid64 = -1) {
+                   sdg_cg_info* info, cudaStream_t s, bool singular, bool fp32, int sid64 = -1,
+                   bool cooperative = true) {
   const long long n = h->g.ndof;
   // deflate the kernel in the FP32 iterations when it is more than the
   // constants (the constants are annihilated exactly by the operator kernel)
@@ -379,7 +389,7 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   // iterations stay single launches); its replacements are one launch too
   // where the FP64 tiles fit (whole)
   const ResPlan& plan = h->res[fp32 ? 1 : 0];
-  const bool resident = !deflate && h->form == 2 && !(h->tile_asked && (fp32 || h->dim == 3)) && !h->profile && plan.state == 1;
+  const bool resident = cooperative && !deflate && h->form == 2 && !(h->tile_asked && (fp32 || h->dim == 3)) && !h->profile && plan.state == 1;
   const bool whole = resident && h->res[0].state == 1;
   // one launch per iteration or less unless asked otherwise or the FP32
   // iteration deflates the kernel
@@ -388,6 +398,8 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
   double* Ap64v[2] = {h->Ap64, fused ? h->Ap64b : h->Ap64};
   float* r32v[2] = {h->r32, fused ? h->r32b : h->r32};
   float* Ap32v[2] = {h->Ap32, fused ? h->Ap32b : h->Ap32};
+  // the same solve from its start without cooperative launches
+  auto with_launches = [&] { return solve_reliable(h, op, b, x, rtol, sid, info, s, singular, fp32, sid64, false); };
   int a64 = 0, updates = 0;
   h->res_seg = 0;  // (not 0 after a solve that ended with an error: its tags stay taken)
   double floor_res = 0.0;
@@ -396,8 +408,8 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
     rsd.start = start;
     const int rc = take_tags(h, &h->resid_tag, 3u, s, &rsd.tag);
     if (rc != SDG_OK) return rc;
-    SDG_K(h->dim == 2 ? resid_dispatch_2d(h, h->res[0], rsd, s) : resid_dispatch_3d(h, h->res[0], rsd, s));
-    return SDG_OK;
+    return cooperative_launch(h, h->dim == 2 ? resid_dispatch_2d(h, h->res[0], rsd, s)
+                                             : resid_dispatch_3d(h, h->res[0], rsd, s));
   };
   if (whole) {
     rsd.b = b;
@@ -418,6 +430,7 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
     rsd.delta = fp32 ? delta : 0.0;
     rsd.maxit = h->maxit;
     int rc = resid(1);
+    if (rc == kRefused) return with_launches();
     h->st_host[sid].iter = 0;
     if (rc == SDG_OK) rc = resident_sync(h, sid, s);
     if (rc != SDG_OK) return rc;
@@ -528,16 +541,23 @@ int solve_reliable(sdg_handle* h, const Op& op, const double* b, double* x, doub
     if (resident) {
       rc = fp32 ? cg_resident<float>(h, op, plan, h->x32, r32v, h->p32, Ap32v, sid, s, cap, delta2)
                 : cg_resident<double>(h, op, plan, x, r64v, h->p64, Ap64v, sid, s, cap, delta2);
+      // (x is as it was given until the first segment has run)
+      if (rc == kRefused && it_now == 0 && updates == 0) return with_launches();
       if (rc == SDG_OK && !whole) rc = resident_sync(h, sid, s);
     } else
       rc = fp32 ? cg_loop<float>(h, op, h->x32, r32v, h->p32, Ap32v, sid, s, fused, deflate, cap)
                 : cg_loop<double>(h, op, x, r64v, h->p64, Ap64v, sid, s, fused, false, cap);
-    if (rc != SDG_OK) return rc;
-    if (whole) {
+    if (rc == SDG_OK && whole) {
       // residual replacement behind the segment, one round trip for both
       rc = resid(0);
       if (rc == SDG_OK) rc = resident_sync(h, sid, s);
-      if (rc != SDG_OK) return rc;
+    }
+    if (rc == kRefused) {
+      set_err("a cooperative launch was refused in the middle of a solve%s", "");
+      rc = SDG_ERR_CUDA;
+    }
+    if (rc != SDG_OK) return rc;
+    if (whole) {
       ++a64;
       ++updates;
       log_update(updates);
