@@ -793,7 +793,13 @@ __global__ void __launch_bounds__(Tile<DIM, N1, TV>::THREADS, (apply_min_blocks<
       yp[k] = s_out[e * ES + row * RS + l1];
       pp[k] = s_in[e * ES + row * RS + l1];
     }
-    reinterpret_cast<V*>(a.y)[(size_t)ge * NV + off] = yv;
+    // A plain apply streams its output (first to leave L2), so that it displaces
+    // none of the caller's inputs: 256 x 256 cells, N = 7, FP32, three input and
+    // two output vectors in turn (84 MB): 20.52 us wherever they lie, against
+    // 20.56 to 21.70 us over 15 placements with plain stores.
+    V* const yo = reinterpret_cast<V*>(a.y) + (size_t)ge * NV + off;
+    if (fuse) *yo = yv;
+    else __stcs(yo, yv);
     if (fuse) {
 #pragma unroll
       for (int k = 0; k < VW; ++k) {
