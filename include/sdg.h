@@ -152,7 +152,10 @@ int sdg_destroy(sdg_handle* h);
  *              residual is 7e-10).
  *   SDG_MIXED: iterations and operator applications in FP32; the dot
  *              products are summed as compensated FP32 pairs per thread and
- *              block and finished in FP64; the FP32 correction is folded into
+ *              block and finished in FP64, in cooperative launches
+ *              (sdg_set_iteration_form) in FP32 pairs of about 46 bits, whose
+ *              alpha and beta are within one FP32 rounding of the exact ones
+ *              too; the FP32 correction is folded into
  *              the FP64 solution and the residual replaced whenever the FP32
  *              residual has dropped by the factor delta since the last
  *              replacement (or after max(2000, iterations/8) FP32

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
   for (int k = 0;; ++k) {
     const unsigned tag = a.tag + (unsigned)k;
     unsigned long long* hw = a.halo + (size_t)(k & 1) * a.ndof;
-    // sums: plain along a line (N1 terms), float pairs across lines
+    // sums: compensated term by term along a line, float pairs across lines
     F2 s_pa{0.0f, 0.0f}, s_rr{0.0f, 0.0f}, s_ra{0.0f, 0.0f}, s_aa{0.0f, 0.0f};
 
     // ---- r -= alpha Ap, x += alpha p, p = r + beta p; r.r; boundary lines
@@ -263,7 +263,6 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
       for (int u = 0; u < 2; ++u)
         if (j >= AR) B::load_row(s_ap, slot[u] >= 0 ? aplace(j + u) : 0, lam, av[u]);
       // r of the two rounds (av: r's new values from here on)
-      float rr[2] = {0.0f, 0.0f};
 #pragma unroll
       for (int q = 0; q < R; q += 2) {
         if (j != q) continue;
@@ -282,13 +281,14 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
         const int e = slot[u] & 0xffff;
         float po[N1];
         B::load_row(s_p, e, lam, po);
+        KDot<float> rr;
 #pragma unroll
         for (int m = 0; m < N1; ++m) {
           xv[u][m] = fmaf(alpha, po[m], xv[u][m]);
           po[m] = fmaf(beta, po[m], av[u][m]);
-          rr[u] = fmaf(av[u][m], av[u][m], rr[u]);
+          rr.add(av[u][m], av[u][m]);
         }
-        s_rr = f2_add(s_rr, F2{rr[u], 0.0f});
+        s_rr = f2_add(s_rr, pair(rr));
         B::store_row(s_p, e, lam, po);
         if (slot[u] & 0x10000) {
           if constexpr (N1 % 2 == 0) {
@@ -351,18 +351,18 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
 #pragma unroll
           for (int m = 0; m < N1; ++m) val[m] = fma(a.cmass * wl * s_w[m], xc[m], val[m]);
         }
-        P2 pa(0.0f), ra(0.0f), aa(0.0f);
+        KDot<P2> pa, ra, aa;
 #pragma unroll
         for (int m = 0; m < N1; ++m) {
           val[m] = val[m] + po[m];
-          pa = fma(xc[m], val[m], pa);
-          aa = fma(val[m], val[m], aa);
+          pa.add(xc[m], val[m]);
+          aa.add(val[m], val[m]);
         }
 #pragma unroll
         for (int q = 0; q < R; q += 2) {
           if (j != q) continue;
 #pragma unroll
-          for (int m = 0; m < N1; ++m) ra = fma(P2(r[q][m], r[q + 1][m]), val[m], ra);
+          for (int m = 0; m < N1; ++m) ra.add(P2(r[q][m], r[q + 1][m]), val[m]);
           if (q < AR) {
 #pragma unroll
             for (int m = 0; m < N1; ++m) {
@@ -371,13 +371,13 @@ __global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_cons
             }
           }
         }
-        s_pa = f2_add(s_pa, F2{pa.lo(), 0.0f});
-        s_ra = f2_add(s_ra, F2{ra.lo(), 0.0f});
-        s_aa = f2_add(s_aa, F2{aa.lo(), 0.0f});
+        s_pa = f2_add(s_pa, pair_lo(pa));
+        s_ra = f2_add(s_ra, pair_lo(ra));
+        s_aa = f2_add(s_aa, pair_lo(aa));
         if (two) {
-          s_pa = f2_add(s_pa, F2{pa.hi(), 0.0f});
-          s_ra = f2_add(s_ra, F2{ra.hi(), 0.0f});
-          s_aa = f2_add(s_aa, F2{aa.hi(), 0.0f});
+          s_pa = f2_add(s_pa, pair_hi(pa));
+          s_ra = f2_add(s_ra, pair_hi(ra));
+          s_aa = f2_add(s_aa, pair_hi(aa));
         }
         if (j >= AR) B::store_rows(s_ap, pl0, pl1, lam, val);
       }

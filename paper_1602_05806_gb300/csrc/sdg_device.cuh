@@ -132,6 +132,23 @@ __device__ __forceinline__ P2 operator-(P2 a) { return a * P2(-1.0f); }
 __device__ __forceinline__ P2& operator+=(P2& a, P2 b) { return a = a + b; }
 __device__ __forceinline__ P2& operator-=(P2& a, P2 b) { return a = a - b; }
 
+// A compensated (Kahan) dot product: the sum and what it still lacks, as the
+// two-launch iteration forms its sums.  T = float, or P2 for two at once.
+template <typename T>
+struct KDot {
+  T s, e;
+  __device__ __forceinline__ KDot() : s(0.0f), e(0.0f) {}
+  __device__ __forceinline__ void add(T a, T b) {
+    const T y = fma(a, b, e);
+    const T t = s + y;
+    e = y - (t - s);
+    s = t;
+  }
+};
+__device__ __forceinline__ F2 pair(const KDot<float>& d) { return F2{d.s, d.e}; }
+__device__ __forceinline__ F2 pair_lo(const KDot<P2>& d) { return F2{d.s.lo(), d.e.lo()}; }
+__device__ __forceinline__ F2 pair_hi(const KDot<P2>& d) { return F2{d.s.hi(), d.e.hi()}; }
+
 // Sum K float pairs over the block; totals (as doubles) in every thread.
 // Warps and then warp 0 add pairs with TwoSum; only the block total is
 // converted to FP64 (one thread).  s_red: at least 32*K doubles.
