@@ -369,14 +369,13 @@ cudaError_t pending_x(float* x, const float* p, long long n, SolverState* st, cu
 cudaError_t kernel_restore(const sdg_handle* h, double* x, const double* x0, cudaStream_t s, int* launches);
 
 // ---- line-wise stage kernels (sdg_lines_*.cu) -------------------------------
-// out = base + scale (perpendicular weights, if weights) (K a + s (J K J) b)
-// along d, s = 1 (plus) or -1; a, b read from the element sa, sb away along d
-// (a2 set: a, b stand for c1 a + c2 a2, c1 b + c2 b2); st: the sum of the
-// outputs goes to st->red[0].
+// out = base + scale D (R a + s L b) along d, s = 1 (plus) or -1, D: the
+// perpendicular weights (weights) or 1 / w along d; a, b read from the element
+// sa, sb away along d (a2 set: a, b stand for c1 a + c2 a2, c1 b + c2 b2); st:
+// the sum of the outputs goes to st->red[0].
 struct PairArgs {
   int d;
-  const double* K;   // n1 x n1, host
-  const double* K2;  // weights: J K J as computed (term by term form)
+  const double *R, *L;  // n1 x n1, host; L = J R J (J: reversal) but for rounding
   bool plus, weights;
   const double *a, *b;
   int sa, sb;

@@ -693,22 +693,14 @@ namespace {
 cudaError_t pair_line(const sdg_handle* h, const PairArgs& a, cudaStream_t s) {
   return h->dim == 2 ? pair_dispatch_2d(h, a, s) : pair_dispatch_3d(h, a, s);
 }
-// The matrix K of a pair transform K a + s (J K J) b from R and L = J R J,
-// the mean of the two computed ones (each carries the rounding of its own
-// quadrature), rows scaled by 1 / w.
-void pair_matrix(const sdg_handle* h, const double* R, const double* L, double* out) {
-  const int n1 = h->g.n1, last = n1 * n1 - 1;
-  for (int i = 0; i <= last; ++i) out[i] = 0.5 * (R[i] + L[last - i]) / h->basis.w[i / n1];
-}
 }  // namespace
 
 // M^-1 (M^L in[e-1] + M^R in[e]) along d (Eq. l2forward), M^L = J M^R J
 cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
-  double K[kMaxN1 * kMaxN1];
-  pair_matrix(h, h->basis.MR, h->basis.ML, K);
   PairArgs a{};
   a.d = d;
-  a.K = K;
+  a.R = h->basis.MR;
+  a.L = h->basis.ML;
   a.plus = true;
   a.a = a.b = in;
   a.sb = -1;
@@ -718,11 +710,10 @@ cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double*
 }
 // M^-1 (M^L in[e] + M^R in[e+1]) along d (Eq. l2backward)
 cudaError_t k_main_to_dual(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
-  double K[kMaxN1 * kMaxN1];
-  pair_matrix(h, h->basis.MR, h->basis.ML, K);
   PairArgs a{};
   a.d = d;
-  a.K = K;
+  a.R = h->basis.MR;
+  a.L = h->basis.ML;
   a.plus = true;
   a.a = a.b = in;
   a.sa = 1;
@@ -752,8 +743,8 @@ cudaError_t k_divergence(const sdg_handle* h, const double* const* U, const doub
   for (int d = 0; d < h->dim; ++d) {
     PairArgs a{};
     a.d = d;
-    a.K = h->basis.Rb;
-    a.K2 = h->basis.Lb;
+    a.R = h->basis.Rb;
+    a.L = h->basis.Lb;
     a.weights = true;
     a.a = a.b = U[d];
     a.sb = -1;
@@ -774,12 +765,11 @@ cudaError_t k_shift(double* x, long long n, const SolverState* st, int slot, dou
 // U*_d - (dt/dx_d) M^-1 (R~ q[e+1] - L~ q[e]) (Eq. LOvelocityU), L~ = J R~ J
 cudaError_t k_velocity_update(const sdg_handle* h, const double* const* Ustar, const double* Pn,
                               const double* Po, double* const* U, cudaStream_t s) {
-  double K[kMaxN1 * kMaxN1];
-  pair_matrix(h, h->basis.Rt, h->basis.Lt, K);
   for (int d = 0; d < h->dim; ++d) {
     PairArgs a{};
     a.d = d;
-    a.K = K;
+    a.R = h->basis.Rt;
+    a.L = h->basis.Lt;
     a.a = a.b = Pn;
     a.sa = 1;
     if (h->theta != 1.0) {  // q = theta Pn + (1 - theta) Po

@@ -12,7 +12,12 @@
 //     n^2 instead of 2 n^2 multiply-adds per line.  (Not the divergence: its
 //     terms cancel to 1e-6 and less, and the sums and differences of a and c
 //     are two more roundings of each: 3.6e-11 of a right-hand side on 48^3
-//     cells, N = 4, against 1.9e-11 term by term, for 0.2 of 4.9 ms);
+//     cells, N = 4, against 1.9e-11 term by term, for 0.2 of 4.9 ms.  And not
+//     for n = 2, where those two roundings count: errors against extended
+//     precision 1.2 to 1.5 times those of the term by term form in the
+//     projections and 1.0 to 1.4 times in the velocity update's gradient,
+//     against 0.5 to 1.1 times for n >= 3, where on the mean over degrees,
+//     rough and smooth data they are 0.94 and 0.86 times as large);
 //   * the volume term of the convection, an anti-centrosymmetric matrix,
 //     splits into two blocks of (n/2)^2.
 #pragma once
@@ -81,19 +86,19 @@ __device__ __forceinline__ void pair_apply(const PairMat<N1>& k, const double (&
   if constexpr (N1 % 2) y[H] = yE[H];  // row H of K a + s J K J b is K_H (a + s c)
 }
 
-// K and J K J themselves, for the term by term form.
+// R and -s L themselves, for the term by term form.
 template <int N1>
 struct PairFull {
   double A[N1 * N1], B[N1 * N1];
-  void fill(const double* K, const double* K2) {
+  void fill(const double* R, const double* L, bool plus) {
     for (int i = 0; i < N1 * N1; ++i) {
-      A[i] = K[i];
-      B[i] = K2[i];
+      A[i] = R[i];
+      B[i] = plus ? -L[i] : L[i];
     }
   }
 };
 
-// y = K a - K2 b
+// y = A a - B b
 template <int N1>
 __device__ __forceinline__ void full_apply(const PairFull<N1>& k, const double (&a)[N1], const double (&b)[N1],
                                            double (&y)[N1]) {
@@ -109,10 +114,14 @@ __device__ __forceinline__ void full_apply(const PairFull<N1>& k, const double (
   }
 }
 
+// the term by term form: the divergence (W) and, for accuracy, n = 2
+template <int N1, bool W>
+constexpr bool pair_full() { return W || N1 == 2; }
+
 template <int N1, bool W>
 struct PairParams {
-  typename std::conditional<W, PairFull<N1>, PairMat<N1>>::type k;
-  double w[N1];
+  typename std::conditional<pair_full<N1, W>(), PairFull<N1>, PairMat<N1>>::type k;
+  double w[N1];        // W: weights; term by term otherwise: 1 / w
   LineGeo g;
   const double* a;     // multiplied by K, from element e + sa
   const double* b;     // multiplied by s J K J, from element e + sb
@@ -128,8 +137,7 @@ struct PairParams {
   double* partials;
 };
 
-// out = base + scale (K a + s (J K J) b); W: weights perpendicular to d, s = -1,
-// term by term
+// out = base + scale D (R a + s L b); W: s = -1, D the weights perpendicular to d
 template <int DIM, int N1, bool PLUS, bool W, bool MIX>
 __global__ void __launch_bounds__(256) k_pair_line(const __grid_constant__ PairParams<N1, W> p) {
   constexpr int LINES = DIM == 2 ? N1 : N1 * N1, NPE = LINES * N1;
@@ -168,13 +176,14 @@ __global__ void __launch_bounds__(256) k_pair_line(const __grid_constant__ PairP
         b[q] = fma(p.c1, b[q], p.c2 * p.b2[ib + q * st]);
       }
     }
-    if constexpr (W) full_apply<N1>(p.k, a, b, y);
+    if constexpr (pair_full<N1, W>()) full_apply<N1>(p.k, a, b, y);
     else pair_apply<N1, PLUS>(p.k, a, b, y);
     double f = p.scale;
     if (W) f *= DIM == 2 ? s_w[lam] : s_w[q0] * s_w[q1];
 #pragma unroll
     for (int m = 0; m < N1; ++m) {
-      const double v = p.base ? fma(f, y[m], p.base[io + m * st]) : f * y[m];
+      const double fm = pair_full<N1, W>() && !W ? f * p.w[m] : f;
+      const double v = p.base ? fma(fm, y[m], p.base[io + m * st]) : fm * y[m];
       p.out[io + m * st] = v;
       sum += v;
     }
@@ -340,9 +349,17 @@ inline LineGeo line_geo(const Geo& g, int d) {
 template <int DIM, int N1, bool W>
 cudaError_t launch_pair_w(const sdg_handle* h, const PairArgs& in, cudaStream_t s) {
   PairParams<N1, W> p;
-  if constexpr (W) p.k.fill(in.K, in.K2);
-  else p.k.fill(in.K);
-  for (int i = 0; i < N1; ++i) p.w[i] = h->basis.w[i];
+  const double* w = h->basis.w;
+  if constexpr (pair_full<N1, W>()) {
+    p.k.fill(in.R, in.L, in.plus);
+  } else {
+    // the mean of the two computed matrices (each carries the rounding of its
+    // own quadrature), rows scaled by 1 / w
+    double K[N1 * N1];
+    for (int i = 0; i < N1 * N1; ++i) K[i] = 0.5 * (in.R[i] + in.L[N1 * N1 - 1 - i]) / w[i / N1];
+    p.k.fill(K);
+  }
+  for (int i = 0; i < N1; ++i) p.w[i] = W ? w[i] : 1.0 / w[i];
   p.g = line_geo(h->g, in.d);
   p.a = in.a;
   p.b = in.b;
