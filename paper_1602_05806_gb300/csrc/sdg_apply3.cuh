@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T, N1>
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ring = reinterpret_cast<T*>(smem_raw);  // 3 planes: 3 * PE * ES
   T* halo = ring + 3 * PE * ES;              // face halo, 1 or 2 buffers (L::HB)
-  T* s_out = halo + L::HB * L::HALO_SZ;      // two accumulators: z + x lines, y lines
+  T* s_out = halo + L::HB * L::HALO_SZ;      // accumulators (see March3Smem)
   T* extra = s_out + L::ACCS * PE * ES;            // CG: p_old of the incoming plane and halo / one launch: r_k by ring slot
   T* hpo = extra + PE * ES;
 
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T, N1>
       s_aa = fma(y, y, s_aa);
     }
   };
-  // y = sum of the two accumulators of plane iz, stored; reduced in CG modes
+  // y = sum of the accumulators of plane iz, stored; reduced in CG modes
   auto store_plane = [&](int iz, const T* cur) {
     const int z = z0 + iz;
     const T* rk = extra + (cur - ring);  // ONE
@@ -479,9 +479,7 @@ __global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T, N1>
         if (sx >= VX || sy >= VY) continue;
         const long long ge = ((long long)z * ny + (oy + sy)) * nx + (ox + sx);
         const int si = s * ES + m3_sidx<N1>(q);
-        T y = s_out[PE * ES + si];
-        if constexpr (!AHEAD) y += s_out[2 * PE * ES + si];
-        y += s_out[si];
+        const T y = (s_out[PE * ES + si] + s_out[2 * PE * ES + si]) + s_out[si];
         a.y[(size_t)ge * NPE + q] = y;
         if constexpr (fuse) reduce(y, cur[si], ONE ? rk[si] : T(0));
       }
@@ -578,7 +576,7 @@ __global__ void __launch_bounds__(March3<N1>::THREADS, (march3_min_blocks<T, N1>
     }
     pass(std::integral_constant<int, 0>{}, pm, cur, pp, hx);
     pass(std::integral_constant<int, 1>{}, pm, cur, pp, hx);
-    if constexpr (MODE == 1) {
+    if constexpr (AHEAD && MODE == 1) {
       if (more) load_x(iz + 2);
     }
     __syncthreads();

@@ -32,7 +32,7 @@ namespace sdg {
 
 template <int N1>
 struct BigEl : El2<N1> {
-  static constexpr int NT = big_threads(N1), AR = big_reg_rounds(N1), ROUNDS = big_rounds(N1);
+  static constexpr int NT = kBigThreads, AR = kBigRegRounds, ROUNDS = big_rounds(N1);
   static constexpr int EPW = 32 / N1;       // elements of a warp
   static constexpr int EPR = NT / 32 * EPW;  // elements of a round
 };
@@ -92,7 +92,7 @@ struct BigParams : ResParams<float, 2, N1> {
 };
 
 template <int N1>
-__global__ void __launch_bounds__(big_threads(N1), 1) k_cg_big(const __grid_constant__ BigParams<N1> a) {
+__global__ void __launch_bounds__(kBigThreads, 1) k_cg_big(const __grid_constant__ BigParams<N1> a) {
   using B = BigEl<N1>;
   using TA = ResAcc<float>;
   constexpr int NPE = N1 * N1, NT = B::NT, R = B::ROUNDS, AR = B::AR, EPR = B::EPR;

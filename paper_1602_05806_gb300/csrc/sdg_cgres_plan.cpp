@@ -71,7 +71,7 @@ ResPlan res_plan(const sdg_handle* h, bool fp32) {
   if (best.state == 1 || !fp32 || dim != 2) return best;
   // larger 2D FP32 tiles: as few rounds of lines per thread as possible, then
   // the smallest halo
-  const int epr = big_threads(n1) / 32 * (32 / n1);
+  const int epr = kBigThreads / 32 * (32 / n1);
   for (int ty = 1; ty <= h->g.n[1]; ++ty) {
     if (!canonical(1, ty) || nt[1] > most) continue;
     for (int tx = 1; tx <= h->g.n[0]; ++tx) {
@@ -93,7 +93,7 @@ ResPlan res_plan(const sdg_handle* h, bool fp32) {
       best.nt[1] = nt[1];
       best.nt[2] = 1;
       best.lpt = big_rounds(n1);
-      best.threads = big_threads(n1);
+      best.threads = kBigThreads;
       best.smem = smem;
     }
   }

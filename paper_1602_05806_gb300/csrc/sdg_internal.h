@@ -79,15 +79,15 @@ constexpr int kResMaxSmem = 225 * 1024;  // dynamic shared memory of a CTA (the 
 constexpr int kResMaxN1_3d = 6;          // degrees compiled in 3D (2D: all)
 constexpr int kResMaxCtas = 1024;        // slots of the exchange
 constexpr int kResPolls = 1 << 22;       // polls before a wait gives up (seconds), see sdg_set_wait_limit
-// Large 2D FP32 tiles (sdg_cgbig.cuh), by degree: threads, rounds of lines per
-// thread, rounds whose Ap lives in registers, shared-memory floats per element
-constexpr int big_threads(int) { return 256; }
-constexpr int big_reg_rounds(int) { return 4; }
+// Large 2D FP32 tiles (sdg_cgbig.cuh): threads, rounds of lines whose Ap lives
+// in registers; by degree: rounds per thread, shared-memory floats per element
+constexpr int kBigThreads = 256;
+constexpr int kBigRegRounds = 4;
 constexpr int big_rounds(int n1) { return n1 <= 4 ? 24 : 112 / n1 / 2 * 2; }
 constexpr int big_es(int n1) { return n1 == 8 ? 64 : n1 * (n1 + 1); }  // El2<n1>::ES
 // dynamic shared memory of a tile of te elements with nh halo elements
 constexpr size_t big_smem(int n1, size_t te, size_t nh) {
-  const size_t epr = (size_t)(big_threads(n1) / 32) * (32 / n1), ar = big_reg_rounds(n1);
+  const size_t epr = (size_t)(kBigThreads / 32) * (32 / n1), ar = kBigRegRounds;
   const size_t apn = te > (ar + 2) * epr ? te - ar * epr : 2 * epr;
   return (te + nh + apn) * big_es(n1) * 4 + te * 16 + nh * 4 + 16;
 }
