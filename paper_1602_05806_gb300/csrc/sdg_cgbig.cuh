@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_cg_big(const __grid_constant
 
     // ---- sums, alpha, beta, decisions ----
     F2 v4[4] = {s_pa, s_rr, s_ra, s_aa};
-    unsigned long long* slot = a.slots + (size_t)(k & 1) * kResMaxCtas * 8;
+    unsigned long long* slot = a.slots + (size_t)(k & 1) * a.nslot * 8;
     // (sums formed with an old halo are not posted; s_fail is the same for all
     // threads here, the fetch being behind a barrier)
     if (!s_fail) {

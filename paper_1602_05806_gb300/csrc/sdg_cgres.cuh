@@ -67,7 +67,8 @@ struct ResParams {
   T* ap[2];
   T* x;
   SolverState* st;
-  unsigned long long* slots;  // [2 parities][kResMaxCtas][4 sums][2 words]
+  unsigned long long* slots;  // [2 parities][nslot][4 sums][2 words]
+  int nslot;
   unsigned long long* halo;   // [2 parities][ndof] words (FP64: pairs of them)
   long long ndof;
   unsigned tag;               // exchange k of this launch carries tag + k
@@ -647,7 +648,7 @@ __global__ void __launch_bounds__(res_max_threads<T>(), 1) k_cg_res(const __grid
       }
     }
     A v4[4] = {TA::value(d_pa), TA::value(d_rr), TA::value(d_ra), TA::value(d_aa)};
-    unsigned long long* slot = a.slots + (size_t)(k & 1) * kResMaxCtas * 8;
+    unsigned long long* slot = a.slots + (size_t)(k & 1) * a.nslot * 8;
     res_post_sums<T>(v4, slot, tag, s_red, s_tot);
     // the neighbours' Ap for the next update, published before their sums
     bool fail = NH > 0 && !res_fetch<T, NPE>(s_ah, s_hel, NH, hout, tag, a.polls);
@@ -708,6 +709,7 @@ void fill_res_params(const sdg_handle* h, const ResPlan& pl, const ResArgs<T>& i
   p.x = in.x;
   p.st = in.st;
   p.slots = h->res_slots;
+  p.nslot = h->res_ctas;
   p.halo = h->res_halo;
   p.ndof = h->g.ndof;
   p.tag = in.tag;

@@ -38,7 +38,8 @@ struct ResidParams {
   int kd;               // 0: nothing to project
   double ncell, inv_ncell;
   SolverState* st;
-  unsigned long long* slots;  // [2 parities][kResMaxCtas][16 sums][2 words]
+  unsigned long long* slots;  // [2 parities][nslot][16 sums][2 words]
+  int nslot;
   unsigned tag;
   int polls;            // of a wait before it gives up
   int start;            // 1: start of a solve
@@ -47,10 +48,10 @@ struct ResidParams {
 };
 
 // The sums v[0..15] of every thread of the grid, in s_sum of every CTA.
-// Exchange number `tag`, parity `par`.  All threads of the block call it;
+// Exchange number `tag`, in the words at `slot`.  All threads of the block call it;
 // false (for all of them) when a wait of the CTA ran out: it leaves then.
-__device__ __forceinline__ bool resid_exchange(double (&v)[16], unsigned long long* slots, unsigned tag, int par,
-                                               int limit, double (*s_red)[16], double* s_sum, int* s_fail) {
+__device__ __forceinline__ bool resid_exchange(double (&v)[16], unsigned long long* slot, unsigned tag, int limit,
+                                               double (*s_red)[16], double* s_sum, int* s_fail) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
   // lanes halve the values between them: lane pair 2 i, 2 i + 1 ends with value i
 #pragma unroll
@@ -66,7 +67,6 @@ __device__ __forceinline__ bool resid_exchange(double (&v)[16], unsigned long lo
   if (!(lane & 1)) s_red[wid][lane >> 1] = v[0];
   __syncthreads();
   const int c = lane & 15, h2 = lane >> 4;
-  unsigned long long* slot = slots + (size_t)par * kResMaxCtas * 32;
   if (wid == 0) {
     double t = 0.0;
     for (int w = h2; w < nw; w += 2) t += s_red[w][c];
@@ -250,7 +250,8 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
   auto give_up = [&] {
     if (tid == 0) st->wait_failed = 1;
   };
-  if (!resid_exchange(v, a.slots, a.tag, 0, a.polls, s_red, s_sum, &s_fail)) return give_up();
+  unsigned long long* const slot1 = a.slots + (size_t)a.nslot * 32;  // the other parity's words
+  if (!resid_exchange(v, a.slots, a.tag, a.polls, s_red, s_sum, &s_fail)) return give_up();
   const double ndof = a.ncell * (double)NPE;
   const double bb = s_sum[2], uu0 = s_sum[4], us = s_sum[3];
   double ss = s_sum[1];
@@ -270,7 +271,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
     for (int i = 0; i < 16; ++i) v[i] = 0.0;
 #pragma unroll
     for (int m = 0; m < N1; ++m) v[0] = fma(r[m], r[m], v[0]);
-    if (!resid_exchange(v, a.slots, a.tag + 1, 1, a.polls, s_red, s_sum, &s_fail)) return give_up();
+    if (!resid_exchange(v, slot1, a.tag + 1, a.polls, s_red, s_sum, &s_fail)) return give_up();
     ss = s_sum[0];
   }
 
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_resid(const __grid_constant__ Res
           if (j < a.kd) v[5 + j] = fma(s_kb[j * NPE + lam * N1 + m], d, v[5 + j]);
       }
     }
-    if (!resid_exchange(v, a.slots, a.tag + 2, 0, a.polls, s_red, s_sum, &s_fail)) return give_up();
+    if (!resid_exchange(v, a.slots, a.tag + 2, a.polls, s_red, s_sum, &s_fail)) return give_up();
     if (act) {
 #pragma unroll
       for (int j = 0; j < kResidMaxKd; ++j) {
@@ -412,7 +413,8 @@ cudaError_t launch_resid_t(const sdg_handle* h, const ResPlan& pl, const ResidAr
   p.ncell = (double)h->g.ncell;
   p.inv_ncell = 1.0 / (double)h->g.ncell;
   p.st = in.st;
-  p.slots = h->res_slots + (size_t)2 * kResMaxCtas * 8;
+  p.slots = h->res_slots + (size_t)2 * h->res_ctas * 8;
+  p.nslot = h->res_ctas;
   p.tag = in.tag;
   p.polls = h->polls;
   p.start = in.start;

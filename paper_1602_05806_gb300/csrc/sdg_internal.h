@@ -77,7 +77,7 @@ constexpr int kProfEvents = 64;  // event pairs per CG batch when profiling
 // grid, chosen once per handle and precision.
 constexpr int kResMaxSmem = 225 * 1024;  // dynamic shared memory of a CTA (the static part stays below 2 KB)
 constexpr int kResMaxN1_3d = 6;          // degrees compiled in 3D (2D: all)
-constexpr int kResMaxCtas = 1024;        // slots of the exchange
+constexpr int kResMaxCtas = 1024;        // CTAs of a plan at most
 constexpr int kResPolls = 1 << 22;       // polls before a wait gives up (seconds), see sdg_set_wait_limit
 // Large 2D FP32 tiles (sdg_cgbig.cuh): threads, rounds of lines whose Ap lives
 // in registers; by degree: rounds per thread, shared-memory floats per element
@@ -190,6 +190,7 @@ struct sdg_handle {
   unsigned long long* res_slots;
   unsigned long long* res_halo;
   size_t res_words;
+  int res_ctas;           // slots of an exchange: CTAs of the larger plan
   unsigned res_tag, res_seg, resid_tag;
   int polls;
   // instrumentation
