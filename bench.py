@@ -39,9 +39,11 @@ METRIC = "pressure-CG GDOF/s & s/time-step, mixed vs FP64 at <=1e-10 rel err; % 
 WORKLOAD = "tg2d_256x256_N7"
 CPU_SAMPLE_CELLS = (32, 32)      # oracle sample: same degree / parameters, 32 x 32 cells
 FLUSH_BYTES = 512 << 20          # > 129 MB L2
-# fused CG operator of the default iteration form (FP32): read r, p_old, x;
+# fused CG operator of the two-launch iteration (FP32): read r, p_old, x;
 # write p, Ap, x (x += alpha p_old of the previous iteration rides along)
 BYTES_PER_DOF_FUSED_F32 = 24
+# an iteration beside its operator: updates of r, x, p, four dot products
+FLOPS_PER_DOF_VECTORS = 14
 
 
 def parse():
@@ -323,6 +325,35 @@ def run_ours(args):
     clocks = sampler.stop()
     step_ms = [a.elapsed_time(b) for a, b in ev]
 
+    # ---- one FP32 iteration of the pressure solve, for its roofline: two capped
+    # solves without replacements in between, the difference of their times over
+    # that of their iterations (the cooperative kernel when a solve counts fewer
+    # launches than iterations, else operator and update launch)
+    x_it = torch.randn(h.shape, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    b_it = torch.empty_like(x_it)
+    h.pressure_apply(x_it, b_it)
+    h.set_mixed_options(1e-6)
+    it_us, it_launches = [], 0
+    for _ in range(4):  # (the first warms up)
+        t = {}
+        for cap in (400, 1600):
+            h.set_options(sdg.SDG_MIXED, 1e-12, 1e-12, cap)
+            xk = torch.zeros_like(b_it)
+            before = h.counters()["launches"]
+            a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(stream)
+            inf = h.pressure_cg(b_it, xk, ok=(sdg.SDG_OK, sdg.SDG_ERR_NOT_CONVERGED))
+            e.record(stream)
+            torch.cuda.synchronize()
+            t[cap] = (a.elapsed_time(e), inf["iters"])
+            it_launches = h.counters()["launches"] - before
+        assert t[400][1] < t[1600][1], t
+        it_us.append(1e3 * (t[1600][0] - t[400][0]) / (t[1600][1] - t[400][1]))
+    it_us = min(it_us[1:])
+    cooperative = it_launches < t[1600][1]
+    h.set_options(sdg.SDG_MIXED, 1e-12, 1e-12)
+    h.set_mixed_options()
+
     # ---- one more step with CUDA events around every launch of the fused
     # FP32 operator (on the launch stream), for its roofline
     h.set_profiling(True)
@@ -337,7 +368,8 @@ def run_ours(args):
     tot_step_ms, p_ms_max, work = reduce_over_ranks(dist, tot_step_ms, p_ms, float(ndof * p_applies), "cuda")
     value = work / (p_ms_max * 1e-3) / 1e9
 
-    # ---- dominant kernel: fused FP32 CG operator (roofline)
+    # ---- rooflines: the iteration of the solves, and the fused FP32 operator
+    # of the two-launch iteration
     peaks, peak_src = measured_peaks()
     n32 = cnt["apply_launches"][1]
     avg_ms = cnt["apply_ms"][1] / n32 if n32 else float("nan")
@@ -351,16 +383,25 @@ def run_ours(args):
     frac_hbm = achieved_gbs / hbm_peak
     frac_alu = achieved_tflops / fp32_peak
     traffic = ncu_traffic()
+    it_tflops = (flops_per_dof + FLOPS_PER_DOF_VECTORS) * ndof / it_us / 1e6
+    roofline = {"bound": "alu", "achieved": it_tflops, "peak": fp32_peak, "unit": "TFLOP/s",
+                "frac": it_tflops / fp32_peak,
+                "kernel": ("k_cg_big<8> (one cooperative launch for all iterations of a segment)" if cooperative else
+                           "k_apply<float,2,8> + k_cg_update<float> (two launches per iteration)")
+                + ", per iteration: difference of two capped solves",
+                "us_per_iteration": it_us, "flops_per_iteration": (flops_per_dof + FLOPS_PER_DOF_VECTORS) * ndof,
+                "peak_source": peak_src + " (152 SM x 128 FP32 lanes x 2 x sm_max_mhz)"}
     if frac_hbm >= frac_alu:
-        roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
+        operator = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                     "frac": frac_hbm, "traffic": traffic}
     else:
-        roofline = {"bound": "alu", "achieved": achieved_tflops, "peak": fp32_peak, "unit": "TFLOP/s",
+        operator = {"bound": "alu", "achieved": achieved_tflops, "peak": fp32_peak, "unit": "TFLOP/s",
                     "frac": frac_alu, "traffic": traffic}
-    roofline.update({"kernel": "k_apply<float,2,8> (fused CG operator: x += alpha p_old, p = r + beta p_old, "
-                               "A p, p.Ap; timed in one extra step with events around each launch)",
+    operator.update({"kernel": "k_apply<float,2,8> (fused CG operator of the two-launch iteration, which profiling "
+                               "runs: x += alpha p_old, p = r + beta p_old, A p, p.Ap; timed in one extra step with "
+                               "events around each launch)",
                      "avg_launch_us": avg_ms * 1e3, "launches_timed": n32,
-                     "peak_source": peak_src + (" (hbm_gbs)" if roofline["bound"] == "hbm"
+                     "peak_source": peak_src + (" (hbm_gbs)" if operator["bound"] == "hbm"
                                                 else " (152 SM x 128 FP32 lanes x 2 x sm_max_mhz)"),
                      "hbm_frac": frac_hbm, "alu_frac": frac_alu,
                      "algorithmic_bytes_per_launch": bytes_per_launch,
@@ -558,7 +599,8 @@ def run_ours(args):
                            "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
                 "pressure_iters_per_step": p_iters, "pressure_ms_total": p_ms,
                 "pressure_true_res_max": max(p_true), "pressure_floor_res": max(p_floor),
-                "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
+                "roofline": roofline, "roofline_two_launch_operator": operator, "cpu_baseline": cpu, "e2e": e2e,
+                "gpu_launches": launches,
                 "clocks": clocks, "fp64": fp64, "accuracy": accuracy, "tg3d": tg3d, "batch": batch}
         print(json.dumps(line), flush=True)
     h.close()

@@ -253,7 +253,8 @@ class Handle:
 
     def set_iteration_form(self, form):
         """0: one launch per CG iteration; 1: operator + update launches, x += alpha p in the update;
-        2 (default): operator + update launches, x += alpha p in the next operator launch."""
+        2 (default): one cooperative launch for many iterations where a tile of elements per SM holds the
+        grid, else operator + update launches, x += alpha p in the next operator launch."""
         check(lib().sdg_set_iteration_form(self.h, int(form)))
 
     def set_wait_limit(self, polls=0):
@@ -261,11 +262,13 @@ class Handle:
         check(lib().sdg_set_wait_limit(self.h, int(polls)))
 
     def set_tile(self, variant):
-        """Tile shape of the 2D FP32 operator (0 base, 1 wide in x, 2 wide in y)."""
+        """Tile shape of the 2D FP32 operator (0 base, 1 wide in x, 2 wide in y) or of the 3D operator; solves
+        of a precision that has the shape then launch that operator for every iteration."""
         check(lib().sdg_set_tile(self.h, int(variant)))
 
     def autotune(self, stream=None):
-        """(chosen tile variant, mean launch time in us of every variant)."""
+        """(chosen tile variant, mean launch time in us of every variant).  The variant serves the operator
+        wherever it is launched."""
         v = ctypes.c_int()
         us = (ctypes.c_double * 3)()
         check(lib().sdg_autotune(self.h, ctypes.byref(v), us, _stream(stream)))
