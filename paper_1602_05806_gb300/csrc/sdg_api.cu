@@ -666,7 +666,6 @@ int pressure_rhs(sdg_handle* h, const double* const* Us, const double* Pold, dou
   for (int d = 0; d < h->dim; ++d) op.s[d] = -(1.0 - h->theta) * h->dt / (h->dx[d] * h->dx[d]);
   SDG_K(apply_plain<double>(h, op, Pold, h->tmp, s));
   SDG_K(k_divergence(h, Us, h->tmp, -1.0, b, st_dev(h, kStMisc), parts(h, kStMisc), s));
-  h->launches += h->dim - 1;  // a launch per direction
   SDG_K(k_shift(b, h->g.ndof, st_dev(h, kStMisc), 0, 1.0 / (double)h->g.ndof, s));
   return SDG_OK;
 }
@@ -1106,7 +1105,6 @@ int sdg_velocity_update(sdg_handle* h, const double* const* Ustar, const double*
                         double* const* U, void* stream) {
   SDG_ARG(h && Ustar && P_new && P_old && U, "bad arguments");
   SDG_K(k_velocity_update(h, Ustar, P_new, P_old, U, S(stream)));
-  h->launches += h->dim - 1;  // a launch per direction
   return SDG_OK;
 }
 
@@ -1160,7 +1158,6 @@ int sdg_step(sdg_handle* h, int nsteps, sdg_step_info* info, void* stream) {
     SDG_K(k_shift(h->Pn, n, st_dev(h, kStMisc), 1, 1.0 / (double)h->g.ncell, s));
     // 7. velocity update with q = theta P^{n+1} + (1-theta) P^n (Eq. LOvelocityU-W)
     SDG_K(k_velocity_update(h, h->Us, h->Pn, h->P, h->U, s));
-    h->launches += h->dim - 1;
     double* t = h->P;
     h->P = h->Pn;
     h->Pn = t;
@@ -1354,7 +1351,6 @@ int sdg_diagnostics(sdg_handle* h, double* kinetic_energy, double* div_norm, voi
   }
   if (div_norm) {
     SDG_K(k_divergence(h, h->U, nullptr, 1.0, h->tmp, st, pa, s));
-    h->launches += h->dim - 1;
     SDG_K(k_norm2(h->tmp, h->g.ndof, st, 3, pa, s));
     SDG_CK(cudaMemcpyAsync(h->st_host + kStMisc, st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
     SDG_CK(cudaStreamSynchronize(s));

@@ -370,24 +370,35 @@ cudaError_t pending_x(float* x, const float* p, long long n, SolverState* st, cu
 cudaError_t kernel_restore(const sdg_handle* h, double* x, const double* x0, cudaStream_t s, int* launches);
 
 // ---- line-wise stage kernels (sdg_lines_*.cu) -------------------------------
-// out = base + scale D (R a + s L b) along d, s = 1 (plus) or -1, D: the
-// perpendicular weights (weights) or 1 / w along d; a, b read from the element
-// sa, sb away along d (a2 set: a, b stand for c1 a + c2 a2, c1 b + c2 b2); st:
-// the sum of the outputs goes to st->red[0].
+// out = base + scale (1 / w) (R a + s L b) along every direction of dir, in one
+// launch: s = 1 (plus) or -1; a, b the lines of x in the elements sa, sb away
+// (x2 set: of c1 x + c2 x2).
 struct PairArgs {
-  int d;
   const double *R, *L;  // n1 x n1, host; L = J R J (J: reversal) but for rounding
-  bool plus, weights;
-  const double *a, *b;
+  bool plus;
+  const double *x, *x2;
   int sa, sb;
-  const double *a2, *b2;
   double c1, c2;
-  const double* base;
+  int ndir;
+  struct {
+    int d;
+    const double* base;  // null: nothing
+    double scale;
+    double* out;
+  } dir[3];
+};
+// out = base + scale sum_d (1/dx_d) M^{perp d} (R-bar U_d[e] - L-bar U_d[e-1]),
+// the sum of out in st->red[0].
+struct DivArgs {
+  const double* const* U;
+  const double* base;  // null: nothing
   double scale;
   double* out;
   SolverState* st;
   double* partials;
 };
+cudaError_t div_dispatch_2d(const sdg_handle* h, const DivArgs& a, cudaStream_t s);
+cudaError_t div_dispatch_3d(const sdg_handle* h, const DivArgs& a, cudaStream_t s);
 cudaError_t pair_dispatch_2d(const sdg_handle* h, const PairArgs& a, cudaStream_t s);
 cudaError_t pair_dispatch_3d(const sdg_handle* h, const PairArgs& a, cudaStream_t s);
 struct ConvArgs {

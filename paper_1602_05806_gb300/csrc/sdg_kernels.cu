@@ -698,27 +698,25 @@ cudaError_t pair_line(const sdg_handle* h, const PairArgs& a, cudaStream_t s) {
 // M^-1 (M^L in[e-1] + M^R in[e]) along d (Eq. l2forward), M^L = J M^R J
 cudaError_t k_dual_to_main(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
   PairArgs a{};
-  a.d = d;
   a.R = h->basis.MR;
   a.L = h->basis.ML;
   a.plus = true;
-  a.a = a.b = in;
+  a.x = in;
   a.sb = -1;
-  a.scale = 1.0;
-  a.out = out;
+  a.ndir = 1;
+  a.dir[0] = {d, nullptr, 1.0, out};
   return pair_line(h, a, s);
 }
 // M^-1 (M^L in[e] + M^R in[e+1]) along d (Eq. l2backward)
 cudaError_t k_main_to_dual(const sdg_handle* h, int d, const double* in, double* out, cudaStream_t s) {
   PairArgs a{};
-  a.d = d;
   a.R = h->basis.MR;
   a.L = h->basis.ML;
   a.plus = true;
-  a.a = a.b = in;
+  a.x = in;
   a.sa = 1;
-  a.scale = 1.0;
-  a.out = out;
+  a.ndir = 1;
+  a.dir[0] = {d, nullptr, 1.0, out};
   return pair_line(h, a, s);
 }
 cudaError_t k_convect_stage(const sdg_handle* h, const double* const* V0, const double* const* V,
@@ -736,27 +734,17 @@ cudaError_t k_mass_rhs(const sdg_handle* h, const double* F, double* b, double* 
   k_mass<<<grid_full(h->g.ndof), kThreads, 0, s>>>(h->g, F, b, x0, h->mats);
   return cudaGetLastError();
 }
-// base + scale sum_d (1/dx_d) M^{perp d} (R-bar U_d[e] - L-bar U_d[e-1]) (Eq. pSDG1), L-bar = J R-bar J;
-// a launch per direction, the last one sums the outputs
+// base + scale sum_d (1/dx_d) M^{perp d} (R-bar U_d[e] - L-bar U_d[e-1]) (Eq. pSDG1)
 cudaError_t k_divergence(const sdg_handle* h, const double* const* U, const double* base, double scale,
                          double* out, SolverState* st, double* partials, cudaStream_t s) {
-  for (int d = 0; d < h->dim; ++d) {
-    PairArgs a{};
-    a.d = d;
-    a.R = h->basis.Rb;
-    a.L = h->basis.Lb;
-    a.weights = true;
-    a.a = a.b = U[d];
-    a.sb = -1;
-    a.base = d == 0 ? base : out;
-    a.scale = scale / h->dx[d];
-    a.out = out;
-    a.st = d == h->dim - 1 ? st : nullptr;
-    a.partials = partials;
-    const cudaError_t e = pair_line(h, a, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  DivArgs a{};
+  a.U = U;
+  a.base = base;
+  a.scale = scale;
+  a.out = out;
+  a.st = st;
+  a.partials = partials;
+  return h->dim == 2 ? div_dispatch_2d(h, a, s) : div_dispatch_3d(h, a, s);
 }
 cudaError_t k_shift(double* x, long long n, const SolverState* st, int slot, double factor, cudaStream_t s) {
   k_shift_kernel<<<grid_for(n), kThreads, 0, s>>>(x, n, st, slot, factor);
@@ -765,25 +753,19 @@ cudaError_t k_shift(double* x, long long n, const SolverState* st, int slot, dou
 // U*_d - (dt/dx_d) M^-1 (R~ q[e+1] - L~ q[e]) (Eq. LOvelocityU), L~ = J R~ J
 cudaError_t k_velocity_update(const sdg_handle* h, const double* const* Ustar, const double* Pn,
                               const double* Po, double* const* U, cudaStream_t s) {
-  for (int d = 0; d < h->dim; ++d) {
-    PairArgs a{};
-    a.d = d;
-    a.R = h->basis.Rt;
-    a.L = h->basis.Lt;
-    a.a = a.b = Pn;
-    a.sa = 1;
-    if (h->theta != 1.0) {  // q = theta Pn + (1 - theta) Po
-      a.a2 = a.b2 = Po;
-      a.c1 = h->theta;
-      a.c2 = 1.0 - h->theta;
-    }
-    a.base = Ustar[d];
-    a.scale = -h->dt / h->dx[d];
-    a.out = U[d];
-    const cudaError_t e = pair_line(h, a, s);
-    if (e != cudaSuccess) return e;
+  PairArgs a{};
+  a.R = h->basis.Rt;
+  a.L = h->basis.Lt;
+  a.x = Pn;
+  a.sa = 1;
+  if (h->theta != 1.0) {  // q = theta Pn + (1 - theta) Po
+    a.x2 = Po;
+    a.c1 = h->theta;
+    a.c2 = 1.0 - h->theta;
   }
-  return cudaSuccess;
+  a.ndir = h->dim;
+  for (int d = 0; d < h->dim; ++d) a.dir[d] = {d, Ustar[d], -h->dt / h->dx[d], U[d]};
+  return pair_line(h, a, s);
 }
 cudaError_t k_weighted_sum(const sdg_handle* h, const double* x, const double* y, SolverState* st, int slot,
                            double* partials, cudaStream_t s) {

@@ -22,6 +22,7 @@
 //     splits into two blocks of (n/2)^2.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "sdg_device.cuh"
@@ -114,84 +115,160 @@ __device__ __forceinline__ void full_apply(const PairFull<N1>& k, const double (
   }
 }
 
-// the term by term form: the divergence (W) and, for accuracy, n = 2
-template <int N1, bool W>
-constexpr bool pair_full() { return W || N1 == 2; }
+// the pair transform is formed term by term, for accuracy, for n = 2
+constexpr bool pair_full(int n1) { return n1 == 2; }
 
-template <int N1, bool W>
+template <int N1>
 struct PairParams {
-  typename std::conditional<pair_full<N1, W>(), PairFull<N1>, PairMat<N1>>::type k;
-  double w[N1];        // W: weights; term by term otherwise: 1 / w
-  LineGeo g;
-  const double* a;     // multiplied by K, from element e + sa
-  const double* b;     // multiplied by s J K J, from element e + sb
-  int sa, sb;
-  // MIX: both lines are c1 (a, b) + c2 (a2, b2); read and mixed per direction
-  // rather than once into a buffer, so that the call needs no scratch
-  const double *a2, *b2;
+  typename std::conditional<pair_full(N1), PairFull<N1>, PairMat<N1>>::type k;
+  double wi[N1];         // 1 / w (term by term)
+  int n[3];
+  unsigned nlines;
+  int sa, sb;            // elements along d from which the line multiplied by R (K), by L (J K J) is read
+  // MIX: both lines are of c1 x + c2 x2; read and mixed per direction rather
+  // than once into a buffer, so that the call needs no scratch
+  const double *x, *x2;
   double c1, c2;
-  const double* base;  // what the result is added to (null: nothing)
-  double scale;
+  struct Dir {
+    int d, st;           // direction, node stride along it
+    const double* base;  // what the result is added to (null: nothing)
+    double scale;
+    double* out;
+  } dir[3];              // by blockIdx.y
+};
+
+// out = base + scale (1 / w) (R a + s L b) along a direction, a and b lines of x
+template <int DIM, int N1, bool PLUS, bool MIX>
+__global__ void __launch_bounds__(256) k_pair_line(const __grid_constant__ PairParams<N1> p) {
+  constexpr int LINES = DIM == 2 ? N1 : N1 * N1, NPE = LINES * N1;
+  const auto& q = p.dir[blockIdx.y];
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= p.nlines) return;
+  const unsigned el = t / LINES;
+  const int lam = (int)(t - el * LINES);
+  const int q0 = lam % N1, q1 = lam / N1;
+  const int lb = DIM == 2 ? (q.d == 0 ? lam * N1 : lam)
+                          : (q.d == 0 ? lam * N1 : q.d == 1 ? q0 + q1 * N1 * N1 : lam);
+  // the neighbours along d
+  const unsigned nx = p.n[0], ny = p.n[1];
+  const unsigned ex = el % nx, ey = (el / nx) % ny;
+  const int pos = q.d == 0 ? (int)ex : q.d == 1 ? (int)ey : (int)(el / (nx * ny));
+  const long long str = q.d == 0 ? 1 : q.d == 1 ? (long long)nx : (long long)nx * ny;
+  const int nd = p.n[q.d];
+  auto nb = [&](int s) -> size_t {
+    long long e = (long long)el + s * str;
+    if (s < 0 && pos == 0) e += nd * str;
+    if (s > 0 && pos == nd - 1) e -= nd * str;
+    return (size_t)e * NPE + lb;
+  };
+  const size_t ia = nb(p.sa), ib = nb(p.sb);
+  const size_t io = (size_t)el * NPE + lb;
+  const int st = q.st;
+  double a[N1], b[N1], y[N1];
+#pragma unroll
+  for (int k = 0; k < N1; ++k) {
+    a[k] = p.x[ia + k * st];
+    b[k] = p.x[ib + k * st];
+    if (MIX) {
+      a[k] = fma(p.c1, a[k], p.c2 * p.x2[ia + k * st]);
+      b[k] = fma(p.c1, b[k], p.c2 * p.x2[ib + k * st]);
+    }
+  }
+  if constexpr (pair_full(N1)) full_apply<N1>(p.k, a, b, y);
+  else pair_apply<N1, PLUS>(p.k, a, b, y);
+#pragma unroll
+  for (int m = 0; m < N1; ++m) {
+    const double f = pair_full(N1) ? q.scale * p.wi[m] : q.scale;
+    q.out[io + m * st] = q.base ? fma(f, y[m], q.base[io + m * st]) : f * y[m];
+  }
+}
+
+// ---- divergence -------------------------------------------------------------
+// out = base + sum_d f_d M^{perp d} (R U_d[e] - L U_d[e-1]), and the sum of out
+// into st->red[0].  A CTA takes runs of G elements and adds the directions up
+// in shared memory (rows of N1 values padded to an odd length), so that base
+// and out move once.  A launch per direction, with the sums through out, costs
+// a launch latency each: right-hand side on 8 x 8 cells, N = 3, 29.7 instead of
+// 24.7 us, on 64 x 64, N = 5, 43.6 instead of 37.0, on 48^3, N = 4, 2 % more.
+template <int N1>
+struct DivParams {
+  PairFull<N1> k;
+  double w[N1];
+  int n[3];
+  unsigned ncell;
+  int G;
+  const double* U[3];
+  double f[3];
+  const double* base;  // null: nothing
   double* out;
-  SolverState* st;     // sum of the outputs into st->red[0] (null: none)
+  SolverState* st;
   double* partials;
 };
 
-// out = base + scale D (R a + s L b); W: s = -1, D the weights perpendicular to d
-template <int DIM, int N1, bool PLUS, bool W, bool MIX>
-__global__ void __launch_bounds__(256) k_pair_line(const __grid_constant__ PairParams<N1, W> p) {
+template <int DIM, int N1>
+constexpr int div_group() {  // elements of a run at most
+  constexpr int lines = DIM == 2 ? N1 : N1 * N1;
+  return lines >= 256 ? 1 : 256 / lines;
+}
+
+template <int DIM, int N1>
+__global__ void __launch_bounds__(256) k_div_line(const __grid_constant__ DivParams<N1> p) {
   constexpr int LINES = DIM == 2 ? N1 : N1 * N1, NPE = LINES * N1;
+  constexpr int RS = N1 | 1, ES = LINES * RS;
+  __shared__ double s_acc[div_group<DIM, N1>() * ES];
   __shared__ double s_w[N1];
-  if (W && threadIdx.x < N1) s_w[threadIdx.x] = p.w[threadIdx.x];
-  if (W) __syncthreads();
+  const int tid = threadIdx.x, nth = blockDim.x;
+  if (tid < N1) s_w[tid] = p.w[tid];
+  const int es = tid / LINES, lam = tid - es * LINES;
+  const int q0 = lam % N1, q1 = lam / N1;
+  auto at = [](int i) { return i / N1 * RS + i % N1; };  // place of value i of the run
+  const unsigned nrun = (p.ncell + p.G - 1) / p.G;
   double sum = 0.0;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < p.g.nlines; t += gridDim.x * blockDim.x) {
-    const unsigned el = t / LINES;
-    const int lam = (int)(t - el * LINES);
-    const int q0 = lam % N1, q1 = lam / N1;
-    const int lb = DIM == 2 ? (p.g.d == 0 ? lam * N1 : lam)
-                            : (p.g.d == 0 ? lam * N1 : p.g.d == 1 ? q0 + q1 * N1 * N1 : lam);
-    // the neighbours along d
-    const unsigned nx = p.g.n[0], ny = p.g.n[1];
-    const unsigned ex = el % nx, ey = (el / nx) % ny;
-    const int pos = p.g.d == 0 ? (int)ex : p.g.d == 1 ? (int)ey : (int)(el / (nx * ny));
-    const long long str = p.g.d == 0 ? 1 : p.g.d == 1 ? (long long)nx : (long long)nx * ny;
-    const int nd = p.g.n[p.g.d];
-    auto nb = [&](int s) -> size_t {
-      long long e = (long long)el + s * str;
-      if (s < 0 && pos == 0) e += nd * str;
-      if (s > 0 && pos == nd - 1) e -= nd * str;
-      return (size_t)e * NPE + lb;
-    };
-    const size_t ia = nb(p.sa), ib = nb(p.sb);
-    const size_t io = (size_t)el * NPE + lb;
-    const int st = p.g.st;
-    double a[N1], b[N1], y[N1];
+  for (unsigned run = blockIdx.x; run < nrun; run += gridDim.x) {
+    const unsigned e0 = run * p.G;
+    const int ne = min((unsigned)p.G, p.ncell - e0);
+    const size_t g0 = (size_t)e0 * NPE;
+    for (int i = tid; i < ne * NPE; i += nth) s_acc[at(i)] = p.base ? p.base[g0 + i] : 0.0;
+    __syncthreads();
+    const unsigned el = e0 + es;
+    const unsigned nx = p.n[0], ny = p.n[1];
+    const unsigned e[3] = {el % nx, (el / nx) % ny, el / (nx * ny)};
 #pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      a[q] = p.a[ia + q * st];
-      b[q] = p.b[ib + q * st];
-      if (MIX) {
-        a[q] = fma(p.c1, a[q], p.c2 * p.a2[ia + q * st]);
-        b[q] = fma(p.c1, b[q], p.c2 * p.b2[ib + q * st]);
+    for (int d = 0; d < DIM; ++d) {
+      if (es < ne) {
+        constexpr int PS = LINES;  // node stride along z
+        const int st = d == 0 ? 1 : d == 1 ? N1 : PS;
+        const int lb = DIM == 2 ? (d == 0 ? lam * N1 : lam) : (d == 0 ? lam * N1 : d == 1 ? q0 + q1 * N1 * N1 : lam);
+        const size_t str = d == 0 ? 1 : d == 1 ? (size_t)nx : (size_t)nx * ny;
+        const size_t em = e[d] == 0 ? el + (p.n[d] - 1) * str : el - str;
+        const double* U = p.U[d];
+        const size_t ia = (size_t)el * NPE + lb, ib = em * NPE + lb;
+        double a[N1], b[N1], y[N1];
+#pragma unroll
+        for (int k = 0; k < N1; ++k) {
+          a[k] = U[ia + k * st];
+          b[k] = U[ib + k * st];
+        }
+        full_apply<N1>(p.k, a, b, y);
+        const double f = p.f[d] * (DIM == 2 ? s_w[lam] : s_w[q0] * s_w[q1]);
+        // rows hold x-lines: a step along y is a row, along z N1 rows
+        const int sst = d == 0 ? 1 : d == 1 ? RS : N1 * RS;
+        double* s = s_acc + es * ES +
+                    (d == 0 ? lam * RS : DIM == 2 ? lam : d == 1 ? q0 + q1 * N1 * RS : q0 + q1 * RS);
+#pragma unroll
+        for (int m = 0; m < N1; ++m) s[m * sst] = fma(f, y[m], s[m * sst]);
       }
+      __syncthreads();
     }
-    if constexpr (pair_full<N1, W>()) full_apply<N1>(p.k, a, b, y);
-    else pair_apply<N1, PLUS>(p.k, a, b, y);
-    double f = p.scale;
-    if (W) f *= DIM == 2 ? s_w[lam] : s_w[q0] * s_w[q1];
-#pragma unroll
-    for (int m = 0; m < N1; ++m) {
-      const double fm = pair_full<N1, W>() && !W ? f * p.w[m] : f;
-      const double v = p.base ? fma(fm, y[m], p.base[io + m * st]) : fm * y[m];
-      p.out[io + m * st] = v;
+    for (int i = tid; i < ne * NPE; i += nth) {
+      const double v = s_acc[at(i)];
+      p.out[g0 + i] = v;
       sum += v;
     }
+    __syncthreads();
   }
-  if (p.st) {
-    double v1[1] = {sum}, tot[1];
-    if (grid_sum<1>(v1, p.partials, &p.st->counter, tot) && threadIdx.x == 0) p.st->red[0] = tot[0];
-  }
+  double v1[1] = {sum}, tot[1];
+  if (grid_sum<1>(v1, p.partials, &p.st->counter, tot) && tid == 0) p.st->red[0] = tot[0];
 }
 
 // ---- convection -------------------------------------------------------------
@@ -346,11 +423,11 @@ inline LineGeo line_geo(const Geo& g, int d) {
   return q;
 }
 
-template <int DIM, int N1, bool W>
-cudaError_t launch_pair_w(const sdg_handle* h, const PairArgs& in, cudaStream_t s) {
-  PairParams<N1, W> p;
+template <int DIM, int N1>
+cudaError_t launch_pair(const sdg_handle* h, const PairArgs& in, cudaStream_t s) {
+  PairParams<N1> p;
   const double* w = h->basis.w;
-  if constexpr (pair_full<N1, W>()) {
+  if constexpr (pair_full(N1)) {
     p.k.fill(in.R, in.L, in.plus);
   } else {
     // the mean of the two computed matrices (each carries the rounding of its
@@ -359,33 +436,53 @@ cudaError_t launch_pair_w(const sdg_handle* h, const PairArgs& in, cudaStream_t 
     for (int i = 0; i < N1 * N1; ++i) K[i] = 0.5 * (in.R[i] + in.L[N1 * N1 - 1 - i]) / w[i / N1];
     p.k.fill(K);
   }
-  for (int i = 0; i < N1; ++i) p.w[i] = W ? w[i] : 1.0 / w[i];
-  p.g = line_geo(h->g, in.d);
-  p.a = in.a;
-  p.b = in.b;
+  for (int i = 0; i < N1; ++i) p.wi[i] = 1.0 / w[i];
+  for (int k = 0; k < 3; ++k) p.n[k] = h->g.n[k];
+  p.nlines = (unsigned)(h->g.ndof / N1);
   p.sa = in.sa;
   p.sb = in.sb;
-  p.a2 = in.a2;
-  p.b2 = in.b2;
+  p.x = in.x;
+  p.x2 = in.x2;
   p.c1 = in.c1;
   p.c2 = in.c2;
-  p.base = in.base;
-  p.scale = in.scale;
-  p.out = in.out;
-  p.st = in.st;
-  p.partials = in.partials;
-  unsigned grid = (p.g.nlines + 255) / 256;
-  if (in.st && grid > (unsigned)kReduceBlocks) grid = kReduceBlocks;
-  if constexpr (W) k_pair_line<DIM, N1, false, true, false><<<grid, 256, 0, s>>>(p);
-  else if (in.plus) k_pair_line<DIM, N1, true, false, false><<<grid, 256, 0, s>>>(p);
-  else if (in.a2) k_pair_line<DIM, N1, false, false, true><<<grid, 256, 0, s>>>(p);
-  else k_pair_line<DIM, N1, false, false, false><<<grid, 256, 0, s>>>(p);
+  for (int k = 0; k < in.ndir; ++k) {
+    const int d = in.dir[k].d;
+    p.dir[k] = {d, line_geo(h->g, d).st, in.dir[k].base, in.dir[k].scale, in.dir[k].out};
+  }
+  // As many threads in a CTA as leave every SM one: on few lines the FP64 pipes
+  // of a few SMs held whole CTAs of 256 while the others idled (projection on
+  // 31 x 21 cells, N = 8: 12.3 us with 23 CTAs, 7.3 us with 184).
+  const unsigned per_sm = (p.nlines * in.ndir + h->nsm - 1) / h->nsm;
+  const unsigned threads = per_sm >= 256 ? 256 : (per_sm + 31) / 32 * 32;
+  const dim3 grid((p.nlines + threads - 1) / threads, in.ndir);
+  if (in.plus) k_pair_line<DIM, N1, true, false><<<grid, threads, 0, s>>>(p);
+  else if (in.x2) k_pair_line<DIM, N1, false, true><<<grid, threads, 0, s>>>(p);
+  else k_pair_line<DIM, N1, false, false><<<grid, threads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
 template <int DIM, int N1>
-cudaError_t launch_pair(const sdg_handle* h, const PairArgs& in, cudaStream_t s) {
-  return in.weights ? launch_pair_w<DIM, N1, true>(h, in, s) : launch_pair_w<DIM, N1, false>(h, in, s);
+cudaError_t launch_div(const sdg_handle* h, const DivArgs& in, cudaStream_t s) {
+  constexpr int LINES = DIM == 2 ? N1 : N1 * N1, G = div_group<DIM, N1>();
+  DivParams<N1> p;
+  p.k.fill(h->basis.Rb, h->basis.Lb, false);
+  for (int i = 0; i < N1; ++i) p.w[i] = h->basis.w[i];
+  for (int k = 0; k < 3; ++k) {
+    p.n[k] = h->g.n[k];
+    p.U[k] = k < DIM ? in.U[k] : nullptr;
+    p.f[k] = k < DIM ? in.scale / h->dx[k] : 0.0;
+  }
+  p.ncell = (unsigned)h->g.ncell;
+  // (as for the pairs: no more elements in a run than leave every SM one)
+  p.G = (int)std::min<long long>(G, (h->g.ncell + h->nsm - 1) / h->nsm);
+  p.base = in.base;
+  p.out = in.out;
+  p.st = in.st;
+  p.partials = in.partials;
+  const long long runs = (h->g.ncell + p.G - 1) / p.G;
+  const int threads = (p.G * LINES + 31) / 32 * 32;
+  k_div_line<DIM, N1><<<(unsigned)std::min<long long>(runs, kReduceBlocks), threads, 0, s>>>(p);
+  return cudaGetLastError();
 }
 
 template <int DIM, int N1>
