@@ -17,12 +17,13 @@
 // passes of an element exchange its values inside the warp, in the element's
 // place of the Ap store, with no block barrier.
 //
-// Measured, us per iteration of the mixed solver, two launches -> here: 40.2
-// -> 26.9 (256 x 256, N = 7), 50.7 -> 32.8 (256 x 256, N = 6), 34.3 -> 22.4
-// (256 x 256, N = 5), 21.5 -> 10.9 (256 x 256, N = 3), 48.0 -> 29.7 (128 x
-// 128, N = 11).  Cycles of the first (52000): update 14400 (of which x 5800),
-// passes 27000, halo 4700, sums, exchange and decisions 6500.  512 threads
-// with one line at a time: 28.4 us; a scalar form with 256 threads: 54 us.
+// Measured, us per iteration of the mixed solver, two launches -> here: 39.2
+// -> 25.6 (256 x 256, N = 7), 47.3 -> 30.9 (256 x 256, N = 6), 30.2 -> 19.9
+// (256 x 256, N = 5), 18.8 -> 9.4 (256 x 256, N = 3), 41.8 -> 25.8 (128 x 128,
+// N = 11).  Cycles of the first, its sums still plain along a line (52000):
+// update 14400 (of which x 5800), passes 27000, halo 4700, sums, exchange and
+// decisions 6500.  512 threads with one line at a time took 1.5 us more, a
+// scalar form with 256 threads twice as long.
 #pragma once
 
 #include "sdg_cgres.cuh"
